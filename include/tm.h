@@ -106,7 +106,9 @@ size_t tm_half_field_bytes(tm_lattice lat, tm_prec prec);
 /* Launch configuration of the hopping kernel for one storage form (a tuning knob; no paper
  * counterpart).  Each output site's 8 hops are shared by 1, 2 or 4 threads (the partial sums
  * are added in a fixed order); more threads per site keep more memory requests in flight on
- * lattices too small to fill the GPU.  The value 3 (TM_HOP_PIPELINED, FP32 and FP16 storage
+ * lattices too small to fill the GPU.  With FP64 storage and 18-real links (computed in 64-bit fixed
+ * point on the integer units, at more than FP64's accuracy) each of these threads is a pair of lanes,
+ * one per projected spin component.  The value 3 (TM_HOP_PIPELINED, FP32 and FP16 storage
  * only) selects one thread per site whose loads of the next hop are issued before the current
  * hop's arithmetic.  The value 5 (TM_HOP_PAIRED, FP32 and FP16 storage only) selects one thread
  * per TWO sites whose FP32 arithmetic runs on packed pairs (one instruction for both sites).
@@ -157,7 +159,7 @@ tm_status tm_apply_D(tm_lattice lat, double *out, const double *in, int flavour,
  * of parity out_parity, from the half field of the other parity (H_eo / H_oe of eq. eo2;
  * M_eo = -kappa H_eo).  in, out: device half fields of precision `prec`, nrhs of them;
  * out must not overlap in.  Links in format `link` (built on first use).  Arithmetic is
- * FP64 for TM_F64 and FP32 otherwise.  The spin projection (1 +- gamma_mu) is applied
+ * FP64 for TM_F64 (with 18-real links: 57-bit fixed point) and FP32 otherwise.  The spin projection (1 +- gamma_mu) is applied
  * before the SU(3) multiply (Sec. 4.1), so each hop multiplies two colour vectors.
  * Errors: TM_ERR_NO_GAUGE, TM_ERR_ARG, TM_ERR_UNSUPPORTED, TM_ERR_CUDA. */
 tm_status tm_apply_hopping_eo(tm_lattice lat, int out_parity, void *out, const void *in,

@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "tm_batch.cuh"
+#include "tm_hop_fx.cuh"
 #include "tm_solver.cuh"
 
 namespace tmq {
@@ -83,17 +84,19 @@ __global__ void plans_init_kernel(Plans L) {
 }
 
 // The batched hopping kernel: the blocks of the listed systems, each computed by the hopping
-// kernels' own body (TPS threads per site, hop_spb(TPS) sites per block) on that system's fields,
+// kernels' own body (TPS threads per site, hop_spb(TPS) sites per block; FP64: the fixed-point body of
+// tm_hop_fx.cuh, two lanes per site) on that system's fields,
 // epilogue coefficients (its mu), CG state and reduction.  serv = 0: the running systems, sloppy
 // storage; serv = 1: the FP64 service of stopped systems, where K4's residual update uses alpha = 1
 // (r = b' - A X from r = b') and the reduction stores ||r||^2 in B.result.  A system that stopped
 // since the list was built (a breakdown in K2) is skipped.
+constexpr int hop_batch_nt(int prec, int tps) { return prec == TM_F64 ? fx_nt(1) : hop_spb(tps) * tps; }
 constexpr int hop_batch_min_blocks(int prec, int nreal, int tps) {
-  return (tps == 1 && (prec == TM_F32 || prec == TM_F16)) ? 512 / hop_spb(1) : 1;  // 8 blocks of 64 (128 registers)
+  return prec == TM_F64 ? 16 * 32 / fx_nt(1) : (tps == 1 && (prec == TM_F32 || prec == TM_F16)) ? 512 / hop_spb(1) : 1;  // 8 blocks of 64 (128 registers)
 }
 
 template <int PREC, int NREAL, bool HAS_Y, int MODE, int TPS>
-__global__ void __launch_bounds__(hop_spb(TPS) * TPS, hop_batch_min_blocks(PREC, NREAL, TPS))
+__global__ void __launch_bounds__(hop_batch_nt(PREC, TPS), hop_batch_min_blocks(PREC, NREAL, TPS))
     hop_batch_kernel(const BatchSys* __restrict__ systems, const CGState* __restrict__ states, Plan plan, int serv,
                      int in_sel, int y_sel, int out_sel, int kk, int out_parity) {
   const int total = plan.start[plan.nlat];
@@ -103,9 +106,14 @@ __global__ void __launch_bounds__(hop_spb(TPS) * TPS, hop_batch_min_blocks(PREC,
     if (serv ? !(S.done && !S.finished) : S.done) continue;  // block-uniform
     const BatchSys& B = systems[m.x];
     const Reduce red{B.partials, B.counters, B.result, B.st, serv ? FIN_STORE : (MODE == 1 ? FIN_CG_ALPHA : FIN_CG_RR)};
-    hop_sites<PREC, NREAL, HAS_Y, MODE, TPS, false, ListBlock, hop_spb(TPS)>(
-        B.g, out_parity, B.links, B.vec[in_sel], 0, B.vec[out_sel], 0, B.vec[y_sel], 0, B.coef[kk],
-        serv ? nullptr : B.st, 1.0, red, ListBlock{m.y, B.nblocks});
+    if constexpr (PREC == TM_F64)
+      hop_sites_fx<HAS_Y, MODE, 1, false>(B.g, out_parity, B.links, B.vec[in_sel], 0, B.vec[out_sel], 0, B.vec[y_sel], 0,
+                                          B.coef[kk], serv ? nullptr : B.st, 1.0, red, ListBlock{m.y, B.nblocks},
+                                          FxArgs{});
+    else
+      hop_sites<PREC, NREAL, HAS_Y, MODE, TPS, false, ListBlock, hop_spb(TPS)>(
+          B.g, out_parity, B.links, B.vec[in_sel], 0, B.vec[out_sel], 0, B.vec[y_sel], 0, B.coef[kk],
+          serv ? nullptr : B.st, 1.0, red, ListBlock{m.y, B.nblocks});
     __syncthreads();  // the body's shared memory is reused by the next block
   }
 }
@@ -288,7 +296,7 @@ template <int PREC, int NREAL, int TPS>
 static tm_status launch_hop_batch(const BatchSys* d_sys, const CGState* d_st, const Plan& plan, int cap, int serv,
                                   int in_sel, int y_sel, int out_sel, int kk, int parity, int mode, bool has_y,
                                   cudaStream_t s) {
-  constexpr int NT = hop_spb(TPS) * TPS;
+  constexpr int NT = hop_batch_nt(PREC, TPS);
 #define TM_GL(HY, MD)                                                                                  \
   {                                                                                                    \
     auto kern = hop_batch_kernel<PREC, NREAL, HY, MD, TPS>;                                            \
@@ -659,7 +667,7 @@ extern "C" tm_status tm_solve_cg_batch(const tm_system* systems, int nsys, const
   };
   std::vector<size_t> offs;
   for (auto& L : lats)
-    for (int q = 0; q < 4; ++q) offs.push_back(add(spinor_bytes_per_site(TM_F64) * L.lat->h));
+    for (int q = 0; q < 4; ++q) offs.push_back(add(fx_field_bytes(L.lat->h)));  // R, Pv, T, W
   for (auto& w : W) {
     const size_t h = w.lat->h;
     for (int q = 0; q < 7; ++q) offs.push_back(add(192 * h));  // be, bo, bp, X, T64, W64, R64

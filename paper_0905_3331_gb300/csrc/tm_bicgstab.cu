@@ -510,8 +510,11 @@ static tm_status schur_apply(const Solver& S, int prec, int nreal, const void* i
   a.out = T;
   a.coef = epi_mdiag_inv_hop(S.mut, S.f);
   a.mode = 0;
+  const bool fx = prec == TM_F64 && nreal == 18;  // T in FX form (tm_dslash_fx.cuh)
+  a.fx.flags = fx ? FX_OUT : 0;
   tm_status st = hop_launch(lat, a, S.s);
   if (st != TM_OK) return st;
+  a.fx.flags = fx ? FX_IN : 0;
   a.out_parity = 1;
   a.in = T;
   a.y = in;
@@ -672,7 +675,9 @@ static tm_status schur_residual(const Solver& S, void* R, const void* X, const v
   a.in = X;
   a.out = T;
   a.coef = epi_mdiag_inv_hop(S.mut, S.f);
+  a.fx.flags = FX_OUT;
   if ((st = hop_launch(lat, a, S.s)) != TM_OK) return st;
+  a.fx.flags = FX_IN;
   a.out_parity = 1;
   a.in = T;
   a.y = X;
@@ -717,7 +722,7 @@ static tm_status solve_one_krylov(tm_lattice lat, double* x, const double* b, co
   // FP64 fields: 0 b_e, 1 b_o, 2 b' (then varphi_o), 3 X, 4 R, 5 T, 6 / 7 scratch of the checks
   void* w[8];
   for (int k = 0; k < 8; ++k) {
-    w[k] = workspace(lat, k, S.hb[TM_F64], &st);
+    w[k] = workspace(lat, k, fx_field_bytes(lat->h), &st);
     if (st != TM_OK) return st;
   }
   void *be = w[0], *bo = w[1], *B = w[2], *X = w[3], *R = w[4], *T = w[5];
@@ -762,8 +767,8 @@ static tm_status solve_one_krylov(tm_lattice lat, double* x, const double* b, co
     v.x = X;
     v.r = R;
     v.T = T;
-    v.p = workspace(lat, 6, S.hb[TM_F64], &st);
-    if (st == TM_OK) v.s = workspace(lat, 7, S.hb[TM_F64], &st);
+    v.p = workspace(lat, 6, fx_field_bytes(lat->h), &st);
+    if (st == TM_OK) v.s = workspace(lat, 7, fx_field_bytes(lat->h), &st);
     if (st == TM_OK) v.rh = workspace(lat, 18, S.hb[TM_F64], &st);
     if (st == TM_OK) v.v = workspace(lat, 19, S.hb[TM_F64], &st);
     if (st == TM_OK) v.t = workspace(lat, 20, S.hb[TM_F64], &st);
@@ -851,7 +856,7 @@ static tm_status solve_one_krylov(tm_lattice lat, double* x, const double* b, co
       // ||varphi_o - Mhat X|| up to the rounding of x_e (2 FP64 hopping launches instead of the
       // Schur residual's 2 followed by the reconstruction's 2)
       double rro = 0.0;
-      if ((st = reconstruct_xo(S, X, be, bo, bfull, x, T, w[6], w[7], &info->true_rel_residual, &rro)) != TM_OK)
+      if ((st = reconstruct_xo(S, X, TM_F64, be, bo, bfull, x, T, w[6], w[7], &info->true_rel_residual, &rro)) != TM_OK)
         return st;
       ++updates;
       if (bi_verbose())
@@ -893,7 +898,7 @@ static tm_status solve_one_krylov(tm_lattice lat, double* x, const double* b, co
   info->reliable_updates = updates;
   info->schur_rel_residual = std::sqrt(rr_true / bb);
   if (!reconstructed &&
-      (st = reconstruct_xo(S, X, be, bo, bfull, x, T, w[6], w[7], &info->true_rel_residual)) != TM_OK)
+      (st = reconstruct_xo(S, X, TM_F64, be, bo, bfull, x, T, w[6], w[7], &info->true_rel_residual)) != TM_OK)
     return st;
   info->status = converged ? TM_OK : TM_ERR_NOT_CONVERGED;
   if (!converged)

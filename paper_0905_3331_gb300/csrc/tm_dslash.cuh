@@ -16,6 +16,7 @@
 // are antiperiodic in time (Sec. 2.4): the hop across t = T-1 <-> 0 is multiplied by -1.
 #pragma once
 
+#include "tm_dslash_fx.cuh"
 #include "tm_internal.cuh"
 
 namespace tmq {
@@ -781,11 +782,16 @@ tm_status hop_launch_t(tm_lattice lat, const HopArgs& a, cudaStream_t s) {
   }
 }
 
+tm_status hop_launch_f64_18(tm_lattice lat, const HopArgs& a, cudaStream_t s);  // tm_hop_fx.cuh
+
 template <int PREC>
 tm_status hop_launch_prec(tm_lattice lat, const HopArgs& a, cudaStream_t s) {
   switch (a.nreal) {
     case 18:
-      return hop_launch_t<PREC, 18>(lat, a, s);
+      if constexpr (PREC == TM_F64)
+        return hop_launch_f64_18(lat, a, s);
+      else
+        return hop_launch_t<PREC, 18>(lat, a, s);
     case 12:
       return hop_launch_t<PREC, 12>(lat, a, s);
     case 8:

@@ -11,7 +11,7 @@
 #include <cstdlib>
 
 #include "tm_doublet.cuh"
-#include "tm_dslash.cuh"
+#include "tm_hop_fx.cuh"
 
 namespace tmq {
 
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(HOP_NT) dhop_kernel(const Geom g, const int ou
 // The same operator with two threads per output site, one per flavour (adjacent lanes).  Both
 // lanes of a pair load the same link (one memory transaction serves the pair), each applies it
 // to its own flavour, and the epilogue takes the partner flavour's sums and site-local input
-// through warp shuffles.  Half the registers of the one-thread form and twice the threads.
+// through warp shuffles.  Half the registers of the one-thread form and twice the threads.  (FP32 storage; FP64 runs dhop_fx_kernel.)
 template <int PREC, int NREAL, bool HAS_Y, int MODE>
 __global__ void __launch_bounds__(HOP_NT) dhop2_kernel(const Geom g, const int out_parity,
                                                        const char* __restrict__ links, const char* in,
@@ -217,6 +217,101 @@ __global__ void __launch_bounds__(HOP_NT) dhop2_kernel(const Geom g, const int o
   }
 }
 
+// The same for FP64 fields and 18-real links: the fixed-point sum of tm_dslash_fx.cuh, four adjacent lanes
+// per output site, one per flavour f and projected spin component q (lane 2 f + q of the site's four;
+// lane q holds spins q and 2 + q).  Lanes of a site load the same link; the flavour mixing takes the
+// partner flavour's values through shuffles.  Bound like the one-flavour kernel (integer issue and
+// latency): it replaces FP64 arithmetic at 1.6 multiply-adds per clock and SM.
+template <bool HAS_Y, int MODE>
+__global__ void __launch_bounds__(HOP_NT, 4) dhop_fx_kernel(const Geom g, const int out_parity,
+                                                            const char* __restrict__ links, const char* in,
+                                                            size_t stride, char* out, size_t out_stride, const char* y,
+                                                            const DCoef co, const CGState* alpha_src, const Reduce red,
+                                                            const int* skip) {
+  __shared__ double sh[HOP_NT / 32];
+  if (skip != nullptr && *skip != 0) return;
+  const int q = threadIdx.x & 1, f = (threadIdx.x >> 1) & 1;
+  const int cb = blockIdx.x * (HOP_NT / 4) + (threadIdx.x >> 2);
+  const bool active = cb < g.h;
+  const char* inf = in + f * stride;
+  const size_t slab = (size_t)FX_LINK_BYTES * g.h;
+  const char* lf = links + (size_t)(out_parity * 4) * slab;
+  const char* lo = links + (size_t)((1 - out_parity) * 4) * slab;
+  cpx<double> acc[6];
+  fx_site<false>(acc, q, active, g, out_parity, cb, inf, inf, lf, lo);
+  const int kq[2] = {3 * q, 6 + 3 * q};
+  cpx<double> yv[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) yv[k] = mk(0.0, 0.0);
+  if (HAS_Y && active) {
+    const double2* p = reinterpret_cast<const double2*>(y + f * stride) + cb;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const double2 t = __ldg(p + (size_t)(kq[k / 3] + k % 3) * g.h);
+      yv[k] = mk(t.x, t.y);
+    }
+  }
+  const int row = co.swap ? 1 - f : f;  // as in dhop2_kernel
+  double nrm = 0.0;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const int ch = k < 3 ? 0 : 1;
+    const cpx<double> ap = mk(__shfl_xor_sync(0xffffffffu, acc[k].re, 2), __shfl_xor_sync(0xffffffffu, acc[k].im, 2));
+    const double(&Qs)[2] = co.Q[ch][row][f], (&Qo)[2] = co.Q[ch][row][1 - f];
+    cpx<double> v = mk(Qs[0], Qs[1]) * acc[k] + mk(Qo[0], Qo[1]) * ap;
+    if (HAS_Y) {
+      const cpx<double> yp = mk(__shfl_xor_sync(0xffffffffu, yv[k].re, 2), __shfl_xor_sync(0xffffffffu, yv[k].im, 2));
+      const double(&Ps)[2] = co.P[ch][row][f], (&Po)[2] = co.P[ch][row][1 - f];
+      v = v + mk(Ps[0], Ps[1]) * yv[k] + mk(Po[0], Po[1]) * yp;
+    }
+    acc[k] = (co.swap && ch == 1) ? mk(-v.re, -v.im) : v;
+  }
+  if (active) {
+    double2* p = reinterpret_cast<double2*>(out + f * out_stride) + cb;
+    const double al = (MODE == 2 && alpha_src) ? alpha_src->alpha : 1.0;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      double2* pk = p + (size_t)(kq[k / 3] + k % 3) * g.h;
+      cpx<double> o = acc[k];
+      if (MODE == 2) {
+        const double2 t = *pk;
+        o = mk(t.x, t.y) - al * o;
+      }
+      if (MODE >= 1) nrm += norm2(o);
+      *pk = make_double2(o.re, o.im);
+    }
+  }
+  if (MODE >= 1) {
+    const double bs = block_sum<HOP_NT>(nrm, sh);
+    grid_reduce<HOP_NT>(red, 0, gridDim.x, blockIdx.x, bs, sh);
+  }
+}
+
+static tm_status dhop_fx_launch(tm_lattice lat, const DHopArgs& a, cudaStream_t s) {
+  const Geom& g = lat->geom;
+  const char* links = static_cast<const char*>(lat->links[TM_F64][link_index(18)]);
+  const char* in = static_cast<const char*>(a.in);
+  const char* y = static_cast<const char*>(a.y);
+  char* out = static_cast<char*>(a.out);
+  const unsigned grid = (unsigned)((g.h + HOP_NT / 4 - 1) / (HOP_NT / 4));
+#define TM_DFX(HY, MM) \
+  dhop_fx_kernel<HY, MM><<<grid, HOP_NT, 0, s>>>(g, a.out_parity, links, in, a.stride, out, a.out_stride, y, a.co, \
+                                                 a.alpha_src, a.red, a.skip)
+  if (!a.y && a.mode == 0)
+    TM_DFX(false, 0);
+  else if (a.y && a.mode == 0)
+    TM_DFX(true, 0);
+  else if (a.y && a.mode == 1)
+    TM_DFX(true, 1);
+  else if (a.y && a.mode == 2)
+    TM_DFX(true, 2);
+  else
+    return set_error(TM_ERR_ARG, "doublet hopping: unsupported epilogue combination");
+#undef TM_DFX
+  count_launch();
+  return cuda_check(cudaGetLastError(), "doublet hopping kernel launch");
+}
+
 static int dhop_threads_per_site() {
   static int v = -1;
   if (v < 0) {
@@ -263,7 +358,7 @@ static tm_status dhop_launch_t(tm_lattice lat, const DHopArgs& a, cudaStream_t s
 tm_status dhop_launch(tm_lattice lat, const DHopArgs& a, cudaStream_t s) {
   tm_status st = ensure_links(lat, a.prec, a.nreal, s);
   if (st != TM_OK) return st;
-  if (a.prec == TM_F64 && a.nreal == 18) return dhop_launch_t<TM_F64, 18>(lat, a, s);
+  if (a.prec == TM_F64 && a.nreal == 18) return dhop_fx_launch(lat, a, s);
   if (a.prec == TM_F32) {
     if (a.nreal == 18) return dhop_launch_t<TM_F32, 18>(lat, a, s);
     if (a.nreal == 12) return dhop_launch_t<TM_F32, 12>(lat, a, s);

@@ -1,5 +1,5 @@
-// tm_dslash_f64.cu -- instantiation of the hopping kernel for TM_F64 spinor storage
-// (all three link formats and every epilogue), compiled as its own translation unit.
+// tm_dslash_f64.cu -- instantiation of the hopping kernel for TM_F64 spinor storage with 12- and
+// 8-real links (FP64 arithmetic, every epilogue), compiled as its own translation unit.
 #include "tm_dslash.cuh"
 
 namespace tmq {

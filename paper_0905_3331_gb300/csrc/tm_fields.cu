@@ -127,7 +127,10 @@ tm_status unpack_full_parity(tm_lattice lat, int prec, double* dst_full, const v
                              cudaStream_t s) {
   const Geom& g = lat->geom;
   const unsigned nb = (unsigned)((g.h + FNT - 1) / FNT);
-  TM_PREC_SWITCH(prec,
+  if (prec == TM_FX)
+    unpack_full_kernel<TM_FX><<<nb, FNT, 0, s>>>(g, static_cast<const char*>(src), dst_full, parity, g5);
+  else
+    TM_PREC_SWITCH(prec,
                  (unpack_full_kernel<P><<<nb, FNT, 0, s>>>(g, static_cast<const char*>(src), dst_full, parity, g5)));
   count_launch();
   return cuda_check(cudaGetLastError(), "unpack kernel");

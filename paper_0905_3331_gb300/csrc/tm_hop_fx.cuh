@@ -1,0 +1,315 @@
+// tm_hop_fx.cuh -- the hopping kernel of FP64 fields and 18-real links: the fixed-point sum of
+// tm_dslash_fx.cuh with the fused epilogues and reductions of tm_dslash.cuh.
+//
+// Two lanes per output site, one per projected spin component (lane q holds spins q and 2 + q of the
+// result), times P direction parts in different warps (P = 1, 2, 4 for 1, 2, 4 "threads per site").
+#pragma once
+
+#include "tm_dslash.cuh"
+
+namespace tmq {
+
+// Sites and threads per block: 64 sites with 128 threads (P = 1), 32 with 128 (2) or 256 (4).
+constexpr int fx_spb(int P) { return P == 1 ? 64 : 32; }
+constexpr int fx_nt(int P) { return fx_spb(P) * 2 * P; }
+
+// The FP64 form of one output site, for the sites whose neighbours have no fixed-point form.  A real
+// call, so that its registers are not the caller's.
+static __device__ __noinline__ void hop_f64_general(const Geom& g, int out_parity, int cb, const char* in,
+                                                    const char* lf, const char* lo, double out[24]) {
+  const SiteCoord c = site_of(g, cb, out_parity);
+  int nb[8];
+  neighbours(g, cb, c, nb);
+  cpx<double> acc[12];
+  hop_part<TM_F64, 18, 1>(acc, g, cb, c, nb, in, lf, lo, link_bytes(TM_F64, 18) * (size_t)g.h, 0);
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    out[2 * k] = acc[k].re;
+    out[2 * k + 1] = acc[k].im;
+  }
+}
+
+// acc = this lane's six components (spins q and 2 + q) of the sum A in FP64, with unit folded in by the
+// caller: real = acc unit.  All lanes of the warp call it (shuffles between the two lanes of a site).
+// in64: the FP64 input, or null.
+__device__ __forceinline__ void fx_finish(const FxAcc& A, int q, bool active, const Geom& g, int out_parity, int cb,
+                                          const char* in64, const char* lf, const char* lo, cpx<double> acc[6],
+                                          double& unit) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {  // the other lane's share of this lane's lower spin 2 + q
+    const fx re = A.s[k].re + __shfl_xor_sync(0xffffffffu, A.o[k].re, 1);
+    const fx im = A.s[k].im + __shfl_xor_sync(0xffffffffu, A.o[k].im, 1);
+    acc[k] = mk<double>((double)A.up[k].re, (double)A.up[k].im);
+    acc[3 + k] = mk<double>((double)re, (double)im);
+  }
+  unit = fx_unit(A.E);
+  if (A.bad && active) {
+    unit = 1.0;
+    if (in64 != nullptr) {
+      double v[24];
+      hop_f64_general(g, out_parity, cb, in64, lf, lo, v);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        acc[k] = mk<double>(v[6 * q + 2 * k], v[6 * q + 2 * k + 1]);
+        acc[3 + k] = mk<double>(v[12 + 6 * q + 2 * k], v[13 + 6 * q + 2 * k]);
+      }
+    } else {
+      const double nan = fx_stored_unit(FX_BAD);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) acc[k] = mk<double>(nan, nan);
+    }
+  }
+}
+
+// The whole sum of a site in its two lanes, as FP64.
+template <bool XIN>
+__device__ __forceinline__ void fx_site(cpx<double> acc[6], int q, bool active, const Geom& g, int out_parity, int cb,
+                                        const char* in, const char* in64, const char* lf, const char* lo) {
+  FxAcc A;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) A.up[k] = A.s[k] = A.o[k] = mk<fx>(0, 0);
+  A.E = 0;
+  A.bad = false;
+  if (active) fx_hops<XIN>(A, q, g, cb, site_of(g, cb, out_parity), in, lf, lo, 0, 4);
+  double unit;
+  fx_finish(A, q, active, g, out_parity, cb, in64, lf, lo, acc, unit);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) acc[k] = unit * acc[k];
+}
+
+// The body: output sites [bid SPB, (bid + 1) SPB) of right-hand side rhs; arguments and modes as
+// hop_sites (tm_dslash.cuh).  XIN: `in` is an FX half field; fxa: the other FX fields.
+template <bool HAS_Y, int MODE, int P, bool XIN, class Blk>
+__device__ __forceinline__ void hop_sites_fx(const Geom g, const int out_parity, const char* __restrict__ links,
+                                             const void* in, size_t in_stride, void* out, size_t out_stride,
+                                             const void* y, size_t y_stride, const EpiCoef coef,
+                                             const CGState* alpha_src, const double alpha_sign, const Reduce red,
+                                             const Blk B, const FxArgs fxa) {
+  constexpr int SPB = fx_spb(P), NT = fx_nt(P);
+  constexpr int WPP = NT / 32 / P;  // warps per part
+  __shared__ double sh[NT / 32];
+  __shared__ fx part_sum[P > 1 ? P * SPB * 2 * 19 : 1];
+  const int warp = threadIdx.x >> 5;
+  const int part = P == 1 ? 0 : warp / WPP;
+  const int lane2 = P == 1 ? (int)threadIdx.x : (warp % WPP) * 32 + (int)(threadIdx.x & 31);  // 2 site + q
+  const int q = lane2 & 1;
+  const int rhs = B.rhs();
+  const int cb = B.bid() * SPB + (lane2 >> 1);
+  const bool active = cb < g.h;
+  FxAcc A;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) A.up[k] = A.s[k] = A.o[k] = mk<fx>(0, 0);
+  A.E = 0;
+  A.bad = false;
+  const char* inr = static_cast<const char*>(in) + (size_t)rhs * in_stride;
+  const size_t slab = (size_t)FX_LINK_BYTES * g.h;
+  const char* lf = links + (size_t)(out_parity * 4) * slab;        // U_mu(x), x of this parity
+  const char* lo = links + (size_t)((1 - out_parity) * 4) * slab;  // U_mu(y), y of the other parity
+  if (active) {
+    const SiteCoord c = site_of(g, cb, out_parity);
+    fx_hops<XIN>(A, q, g, cb, c, inr, lf, lo, part * (4 / P), (part + 1) * (4 / P));
+  }
+  if constexpr (P > 1) {  // the parts' sums meet in part 0, at the largest of their exponents
+    fx* mine = part_sum + (part * SPB * 2 + lane2) * 19;
+    if (part > 0) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        mine[2 * k] = A.up[k].re;
+        mine[2 * k + 1] = A.up[k].im;
+        mine[6 + 2 * k] = A.s[k].re;
+        mine[7 + 2 * k] = A.s[k].im;
+        mine[12 + 2 * k] = A.o[k].re;
+        mine[13 + 2 * k] = A.o[k].im;
+      }
+      mine[18] = A.bad ? -1 : A.E;
+    }
+    __syncthreads();
+    if (part == 0) {
+#pragma unroll
+      for (int p = 1; p < P; ++p) {
+        const fx* o = part_sum + (p * SPB * 2 + lane2) * 19;
+        const int Ep = (int)o[18];
+        if (Ep < 0) {
+          A.bad = true;
+          continue;
+        }
+        const int sa = Ep > A.E ? min(Ep - A.E, 63) : 0, so = A.E > Ep ? min(A.E - Ep, 63) : 0;
+        A.E = max(A.E, Ep);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          A.up[k] = mk<fx>((A.up[k].re >> sa) + (o[2 * k] >> so), (A.up[k].im >> sa) + (o[2 * k + 1] >> so));
+          A.s[k] = mk<fx>((A.s[k].re >> sa) + (o[6 + 2 * k] >> so), (A.s[k].im >> sa) + (o[7 + 2 * k] >> so));
+          A.o[k] = mk<fx>((A.o[k].re >> sa) + (o[12 + 2 * k] >> so), (A.o[k].im >> sa) + (o[13 + 2 * k] >> so));
+        }
+      }
+    }
+  }
+  double nrm = 0.0;
+  if (part == 0) {
+    cpx<double> acc[6];
+    double unit;
+    fx_finish(A, q, active, g, out_parity, cb, XIN ? static_cast<const char*>(fxa.in64) : inr, lf, lo, acc, unit);
+    // epilogue: o_s = D_s (c acc_s + E_s y_s) as (D_s c unit) acc_s + (D_s E_s) y_s; a real D c (every
+    // coefficient set but the inverse site term) takes half the products
+    const double cc = coef.c * unit;
+    const cpx<double> Du = mk(coef.d_up_re, coef.d_up_im), Dl = mk(coef.d_lo_re, coef.d_lo_im);
+    const cpx<double> DCu = mk(coef.d_up_re * cc, coef.d_up_im * cc), DCl = mk(coef.d_lo_re * cc, coef.d_lo_im * cc);
+    const bool real_d = coef.d_up_im == 0.0 && coef.d_lo_im == 0.0;
+    const int kq[2] = {3 * q, 6 + 3 * q};  // this lane's blocks: kq[half] + k
+    cpx<double> o[6];
+    if (HAS_Y) {
+      const cpx<double> Eu = mk(coef.e_up_re, coef.e_up_im), El = mk(coef.e_lo_re, coef.e_lo_im);
+      const cpx<double> DEu = Du * Eu, DEl = Dl * El;
+      cpx<double> yv[6];
+#pragma unroll
+      for (int k = 0; k < 6; ++k) yv[k] = mk(0.0, 0.0);
+      if (active) {
+        const char* yr = static_cast<const char*>(y) + (size_t)rhs * y_stride;
+        if (fxa.flags & FX_Y) {  // uniform
+          const double yu = fx_stored_unit(__ldg(fx_exps(yr, g.h) + cb));
+          const longlong2* p = reinterpret_cast<const longlong2*>(yr) + cb;
+#pragma unroll
+          for (int k = 0; k < 6; ++k) {
+            const longlong2 t = __ldg(p + (size_t)(kq[k / 3] + k % 3) * g.h);
+            yv[k] = mk((double)t.x * yu, (double)t.y * yu);
+          }
+        } else {
+          const double2* p = reinterpret_cast<const double2*>(yr) + cb;
+#pragma unroll
+          for (int k = 0; k < 6; ++k) {
+            const double2 t = __ldg(p + (size_t)(kq[k / 3] + k % 3) * g.h);
+            yv[k] = mk(t.x, t.y);
+          }
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        if (MODE == 3) {
+          const cpx<double> t = cc * acc[k] + (k < 3 ? Eu : El) * yv[k];
+          o[k] = (k < 3 ? Du : Dl) * t;
+          const cpx<double> M = k < 3 ? mk(coef.m_up_re, coef.m_up_im) : mk(coef.m_lo_re, coef.m_lo_im);
+          nrm += norm2(t - M * o[k]);
+        } else {
+          o[k] = (k < 3 ? DEu : DEl) * yv[k];
+        }
+      }
+      if (MODE != 3) {
+        if (real_d) {
+#pragma unroll
+          for (int k = 0; k < 6; ++k) {
+            const double d = k < 3 ? DCu.re : DCl.re;
+            o[k] = mk(fma(d, acc[k].re, o[k].re), fma(d, acc[k].im, o[k].im));
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < 6; ++k) o[k] = o[k] + (k < 3 ? DCu : DCl) * acc[k];
+        }
+      }
+    } else if (real_d) {
+#pragma unroll
+      for (int k = 0; k < 6; ++k) o[k] = (k < 3 ? DCu.re : DCl.re) * acc[k];
+    } else {
+#pragma unroll
+      for (int k = 0; k < 6; ++k) o[k] = (k < 3 ? DCu : DCl) * acc[k];
+    }
+    char* outr = static_cast<char*>(out) + (size_t)rhs * out_stride;
+    if (MODE == 2) {
+      if (active) {
+        const double al = alpha_src ? alpha_sign * alpha_src[rhs].alpha : alpha_sign;
+        double2* p = reinterpret_cast<double2*>(outr) + cb;
+        cpx<double> r[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+          const double2 t = p[(size_t)(kq[k / 3] + k % 3) * g.h];
+          r[k] = mk(t.x, t.y) - al * o[k];
+          nrm += norm2(r[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < 6; ++k) p[(size_t)(kq[k / 3] + k % 3) * g.h] = make_double2(r[k].re, r[k].im);
+      }
+    } else {
+      if (MODE == 1 && active) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) nrm += norm2(o[k]);
+      }
+      if (fxa.flags & FX_OUT) {  // uniform
+        int e = active ? fx_exponent_f64<6>(o) : 0;
+        e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
+        if (active) {
+          longlong2* p = reinterpret_cast<longlong2*>(outr) + cb;
+#pragma unroll
+          for (int k = 0; k < 6; ++k) p[(size_t)(kq[k / 3] + k % 3) * g.h] = fx_pack(o[k], e);
+          if (q == 0) const_cast<int*>(fx_exps(outr, g.h))[cb] = e;
+        }
+      } else if (active) {
+        double2* p = reinterpret_cast<double2*>(outr) + cb;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) p[(size_t)(kq[k / 3] + k % 3) * g.h] = make_double2(o[k].re, o[k].im);
+      }
+    }
+  }
+  if (MODE >= 1) {
+    const double bs = block_sum<NT>(nrm, sh);
+    grid_reduce<NT>(red, rhs, B.nblocks(), B.bid(), bs, sh);
+  }
+}
+
+#ifndef HOP_FX_WARPS
+#define HOP_FX_WARPS 16
+#endif
+// 16 warps per SM (128 registers)
+template <bool HAS_Y, int MODE, int P, bool XIN>
+__global__ void __launch_bounds__(fx_nt(P), HOP_FX_WARPS * 32 / fx_nt(P))
+    hop_fx_kernel(const Geom g, const int out_parity, const char* __restrict__ links, const void* in, size_t in_stride,
+                  void* out, size_t out_stride, const void* y, size_t y_stride, const EpiCoef coef,
+                  const CGState* alpha_src, const double alpha_sign, const Reduce red, const int* skip,
+                  const FxArgs fxa) {
+  pdl_wait();
+  pdl_allow();
+  if (skip != nullptr && *skip != 0) return;
+  hop_sites_fx<HAS_Y, MODE, P, XIN>(g, out_parity, links, in, in_stride, out, out_stride, y, y_stride, coef, alpha_src,
+                                    alpha_sign, red, GridBlock{}, fxa);
+}
+
+template <int P, bool XIN>
+tm_status hop_fx_launch_p(tm_lattice lat, const HopArgs& a, cudaStream_t s) {
+  const Geom& g = lat->geom;
+  constexpr int SPB = fx_spb(P), NT = fx_nt(P);
+  dim3 grid((g.h + SPB - 1) / SPB, a.nrhs);
+  const char* links = static_cast<const char*>(lat->links[TM_F64][link_index(18)]);
+  const bool has_y = a.y != nullptr;
+#define TM_FX_LAUNCH(HY, MD)                                                                                       \
+  launch_pdl(hop_fx_kernel<HY, MD, P, XIN>, grid, dim3(NT), s, g, a.out_parity, links, a.in, a.in_stride, a.out,  \
+             a.out_stride, a.y, a.y_stride, a.coef, a.alpha_src, a.alpha_sign, a.red, a.skip, a.fx)
+  if (!has_y && a.mode == 0)
+    TM_FX_LAUNCH(false, 0);
+  else if (!has_y && a.mode == 1)
+    TM_FX_LAUNCH(false, 1);
+  else if (has_y && a.mode == 0)
+    TM_FX_LAUNCH(true, 0);
+  else if (has_y && a.mode == 1)
+    TM_FX_LAUNCH(true, 1);
+  else if (has_y && a.mode == 2)
+    TM_FX_LAUNCH(true, 2);
+  else if (has_y && a.mode == 3)
+    TM_FX_LAUNCH(true, 3);
+  else
+    return set_error(TM_ERR_ARG, "hopping: unsupported epilogue combination");
+#undef TM_FX_LAUNCH
+  count_launch();
+  return cuda_check(cudaGetLastError(), "hopping kernel launch");
+}
+
+template <bool XIN>
+tm_status hop_fx_launch_t(tm_lattice lat, const HopArgs& a, cudaStream_t s) {
+  switch (lat->hop_tps[TM_F64][link_index(18)]) {
+    case 2:
+      return hop_fx_launch_p<2, XIN>(lat, a, s);
+    case 4:
+      return hop_fx_launch_p<4, XIN>(lat, a, s);
+    default:
+      return hop_fx_launch_p<1, XIN>(lat, a, s);
+  }
+}
+
+}  // namespace tmq

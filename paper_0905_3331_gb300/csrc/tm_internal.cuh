@@ -514,6 +514,28 @@ struct SpinorFmt<TM_DF64> {
   __device__ static __forceinline__ float4 pack(const cpx<float>& z) { return make_float4(z.re, 0.f, z.im, 0.f); }
 };
 
+// FX form of an FP64 half field (tm_dslash_fx.cuh): longlong2 blocks [12][h], int e[h]; a real is
+// V 2^(e - 1081), NaN for e = FX_BAD.  Read-only here.
+constexpr int TM_FX = 4;
+constexpr int FX_BAD = 0x7fff;  // exponent of a site without a fixed-point form
+__device__ __forceinline__ double fx_stored_unit(int e) {
+  return e == FX_BAD ? __longlong_as_double(0x7ff8000000000000ll) : (e == 0 ? 0.0 : __hiloint2double((e - 58) << 20, 0));
+}
+template <>
+struct SpinorFmt<TM_FX> {
+  typedef double real;
+  template <typename R>
+  __device__ static __forceinline__ void load(const void* base, int h, int i, cpx<R> s[12]) {
+    const longlong2* p = static_cast<const longlong2*>(base);
+    const double unit = fx_stored_unit(__ldg(reinterpret_cast<const int*>(p + (size_t)12 * h) + i));
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const longlong2 v = __ldg(p + (size_t)k * h + i);
+      s[k] = mk<R>((R)((double)v.x * unit), (R)((double)v.y * unit));
+    }
+  }
+};
+
 __host__ __device__ inline size_t spinor_bytes_per_site(int prec) {
   return prec == TM_F64 ? 192 : (prec == TM_F32 ? 96 : (prec == TM_F16 ? 52 : 192));
 }
@@ -685,6 +707,39 @@ struct LinkRecon<R, S, 18> {
       for (int b = 0; b < 3; ++b) {
         RawGet<S, BYTES>::put(r, 2 * (3 * a + b), (S)U.m[a][b].re);
         RawGet<S, BYTES>::put(r, 2 * (3 * a + b) + 1, (S)U.m[a][b].im);
+      }
+  }
+};
+
+// FP64 storage with 18 reals: each real u as the integer round(u 2^62) in two signed 32-bit limbs,
+// uh 2^32 + ul (words ul, uh), the operands of the fixed-point hopping sum (tm_dslash_fx.cuh).
+// 2^-63 absolute on matrices whose rows have norm 1; unpack() gives the FP64 number nearest to the
+// stored one, for the kernels with FP64 arithmetic.
+template <>
+struct LinkRecon<double, double, 18> {
+  static constexpr int BYTES = 18 * 8;
+  __device__ static __forceinline__ void unpack(const RawWords<BYTES>& r, Mat3<double>& U) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) U.m[a][b] = mk<double>(get(r, 2 * (3 * a + b)), get(r, 2 * (3 * a + b) + 1));
+  }
+  __device__ static __forceinline__ double get(const RawWords<BYTES>& r, int k) {
+    return fma((double)(int)r.w[2 * k + 1], 0x1p-30, (double)(int)r.w[2 * k] * 0x1p-62);
+  }
+  __device__ static __forceinline__ void put(RawWords<BYTES>& r, int k, double u) {
+    const long long v = __double2ll_rn(u * 0x1p62);
+    const unsigned lo = (unsigned)v, hi = (unsigned)((unsigned long long)v >> 32);
+    r.w[2 * k] = lo;
+    r.w[2 * k + 1] = hi + (lo >> 31);
+  }
+  __device__ static __forceinline__ void pack(RawWords<BYTES>& r, const Mat3<double>& U) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        put(r, 2 * (3 * a + b), U.m[a][b].re);
+        put(r, 2 * (3 * a + b) + 1, U.m[a][b].im);
       }
   }
 };
@@ -1126,8 +1181,8 @@ struct tm_lattice_s {
   int hop_tps[4][3];        // hopping kernel per form (autotuned): threads per site 1, 2, 4, or TM_HOP_PIPELINED
   int hop_tps_forced[4][3]; // set by tm_set_hop_threads: the tuner keeps hands off
   // work space
-  void* ws[32];             // half-field buffers, allocated on demand
-  size_t ws_bytes[32];
+  void* ws[40];             // half-field buffers, allocated on demand
+  size_t ws_bytes[40];
   double* partials;         // reduction partials
   size_t partials_count;
   unsigned* counters;       // reduction counters (zeroed)
@@ -1166,6 +1221,15 @@ tm_status ensure_reduce(tm_lattice lat, size_t nparts, size_t ncounters);
 tm_status ensure_cgstate(tm_lattice lat, size_t n);
 bool is_device_pointer(const void* p);
 
+// FP64 fields in the fixed-point storage form of the FP64 / 18-real hopping launches (FX,
+// tm_dslash_fx.cuh); the FX form of a half field takes fx_field_bytes(h) bytes.
+enum { FX_IN = 1, FX_OUT = 2, FX_Y = 4 };
+struct FxArgs {
+  int flags = 0;               // which of in, out, y are FX half fields
+  const void* in64 = nullptr;  // FX_IN: the FP64 field that in was made from, or null (inside a solver)
+};
+inline size_t fx_field_bytes(size_t h) { return 196 * h; }
+
 // Hopping launch description (one parity, nrhs fields).
 struct HopArgs {
   int out_parity;
@@ -1184,6 +1248,7 @@ struct HopArgs {
   double alpha_sign;
   Reduce red;         // modes 1, 2
   const int* skip;    // if non-null and *skip != 0 the kernel does nothing
+  FxArgs fx;          // FP64 / 18-real launches with one right-hand side
 };
 tm_status hop_launch(tm_lattice lat, const HopArgs& a, cudaStream_t s);
 tm_status hop_launch_dispatch(tm_lattice lat, const HopArgs& a, cudaStream_t s);  // no gauge-copy check
@@ -1204,8 +1269,9 @@ tm_status diag_apply(tm_lattice lat, int prec, void* out, const void* in, int nr
                      double dlr, double dli, cudaStream_t s);
 // Workspace slots: 0..17 CG solver, 22..25 tm_apply_D, 26 staged input, 27 staged output,
 // 28 initial-guess work space, 29 contraction partials, 30 chronological-guess scalars,
-// 31 BiCGstab state; 18..20 BiCGstab vectors; 21 staged correlator matrices.
-enum { WS_GAMMA = 21, WS_APPLY_D = 22, WS_STAGE_IN = 26, WS_STAGE_OUT = 27, WS_X0 = 28, WS_CHRONO = 30, WS_BISTATE = 31 };
+// 31 BiCGstab state; 18..20 BiCGstab vectors; 21 staged correlator matrices; 32 the FX form of an FP64
+// hopping launch's input.
+enum { WS_GAMMA = 21, WS_APPLY_D = 22, WS_STAGE_IN = 26, WS_STAGE_OUT = 27, WS_X0 = 28, WS_CHRONO = 30, WS_BISTATE = 31, WS_FX = 32 };
 // host-buffer staging through workspace slots
 const void* stage_in(tm_lattice lat, int slot, const void* src, size_t bytes, cudaStream_t s, tm_status* st);
 void* stage_out(tm_lattice lat, int slot, void* dst, size_t bytes, tm_status* st);

@@ -116,7 +116,7 @@ extern "C" tm_status tm_solve_normal(tm_lattice lat, void* X, const void* phi, c
   tm_status st = TM_OK;
   void* w[4];
   for (int k = 0; k < 4; ++k) {
-    w[k] = workspace(lat, 4 + k, S.hb[TM_F64], &st);
+    w[k] = workspace(lat, 4 + k, fx_field_bytes(lat->h), &st);
     if (st != TM_OK) return st;
   }
   double bb = 0.0;
@@ -160,7 +160,7 @@ extern "C" tm_status tm_chrono_guess(tm_lattice lat, void* X0, const void* const
   if (n == 0) return cuda_check(cudaStreamSynchronize(s), "synchronise");
   void* w[3];
   for (int k = 0; k < 3; ++k) {
-    w[k] = workspace(lat, 4 + k, S.hb[TM_F64], &st);
+    w[k] = workspace(lat, 4 + k, fx_field_bytes(lat->h), &st);
     if (st != TM_OK) return st;
   }
   void *Achi = w[0], *T = w[1], *W = w[2];

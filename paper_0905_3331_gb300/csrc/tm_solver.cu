@@ -204,13 +204,17 @@ tm_status normal_apply(const Solver& S, int prec, int nreal, const void* in, voi
   a.nreal = nreal;
   a.nrhs = 1;
   a.skip = state ? &state->done : nullptr;
+  // FP64: T and W are FX half fields (tm_dslash_fx.cuh), the form that the FP64 hopping kernel computes in
+  const bool fx = prec == TM_F64 && nreal == 18;
   // K1: T = (M_ee^{-f})^-1 H_eo in
   a.out_parity = 0;
   a.in = in;
   a.out = T;
   a.coef = epi_mdiag_inv_hop(S.mut, -S.f);
   a.mode = 0;
+  a.fx.flags = fx ? FX_OUT : 0;
   if ((st = hop_launch(lat, a, S.s)) != TM_OK) return st;
+  a.fx.flags = fx ? FX_IN | FX_OUT : 0;
   // K2: W = Qhat^{-f} in, <in, A in> = ||W||^2
   a.out_parity = 1;
   a.in = T;
@@ -239,6 +243,7 @@ tm_status normal_apply(const Solver& S, int prec, int nreal, const void* in, voi
   a.out = r;
   a.coef = epi_schur_q(lat->kappa, S.mut, S.f);
   a.mode = 2;
+  a.fx.flags = fx ? FX_IN | FX_Y : 0;
   if (state) {
     a.alpha_src = state;
     a.alpha_sign = 1.0;
@@ -657,22 +662,24 @@ tm_status reconstruct_check(const Solver& S, const void* X, const void* be, cons
   a.in = X;
   a.out = T;
   a.coef = epi_mdiag_inv_hop(S.mut, -S.f);
+  a.fx.flags = FX_OUT;
   if ((st = hop_launch(lat, a, S.s)) != TM_OK) return st;
   a.out_parity = 1;
   a.in = T;
   a.y = X;
   a.out = W;  // x_o
   a.coef = epi_schur_q(lat->kappa, S.mut, -S.f);
+  a.fx.flags = FX_IN | FX_OUT;
   if ((st = hop_launch(lat, a, S.s)) != TM_OK) return st;
-  return reconstruct_xo(S, W, be, bo, bfull, x, T, R, Pv, true_rel, rr_odd);
+  return reconstruct_xo(S, W, TM_FX, be, bo, bfull, x, T, R, Pv, true_rel, rr_odd);
 }
 
-// x_e = (M_ee^f)^-1 (b_e + kappa H_eo x_o) from the odd solution xo, written with xo to the
-// canonical field x; then ||b - M x|| / ||b|| in FP64 (T, R, Pv are FP64 scratch).  Two FP64
+// x_e = (M_ee^f)^-1 (b_e + kappa H_eo x_o) from the odd solution xo (FP64, or FX form: xo_prec), written
+// with xo to the canonical field x; then ||b - M x|| / ||b|| in FP64 (T, R, Pv are FP64 scratch).  Two FP64
 // hopping launches: the first stores x_e and sums the even residual
 // ||b_e + kappa H_eo x_o - M_ee x_e||^2 from the same hopping sum; the second forms
 // (b - M x)_o = b_o - (M_oo x_o - kappa H_oe x_e) and its norm.  R is unused.
-tm_status reconstruct_xo(const Solver& S, const void* xo, const void* be, const void* bo, double bfull, double* x,
+tm_status reconstruct_xo(const Solver& S, const void* xo, int xo_prec, const void* be, const void* bo, double bfull, double* x,
                          void* T, void* R, void* Pv, double* true_rel, double* rr_odd) {
   (void)R;
   tm_lattice lat = S.lat;
@@ -690,6 +697,8 @@ tm_status reconstruct_xo(const Solver& S, const void* xo, const void* be, const 
   a.out = T;  // x_e
   a.coef = epi_scaled_minv(S.mut, S.f, lat->kappa);
   a.mode = 3;
+  const bool xfx = xo_prec == TM_FX;
+  a.fx.flags = (xfx ? FX_IN : 0) | FX_OUT;
   a.red = Reduce{lat->partials, lat->counters, lat->dscalars, nullptr, FIN_STORE};
   if ((st = hop_launch(lat, a, s)) != TM_OK) return st;
   if ((st = cuda_check(cudaMemcpyAsync(Pv, bo, S.hb[TM_F64], cudaMemcpyDeviceToDevice, s), "copy")) != TM_OK)
@@ -700,6 +709,7 @@ tm_status reconstruct_xo(const Solver& S, const void* xo, const void* be, const 
   a.y = W;
   a.out = Pv;
   a.mode = 2;  // Pv -= 1 * (M x)_o
+  a.fx.flags = FX_IN | (xfx ? FX_Y : 0);
   a.alpha_src = nullptr;
   a.alpha_sign = 1.0;
   a.red = Reduce{lat->partials, lat->counters, lat->dscalars + 1, nullptr, FIN_STORE};
@@ -712,8 +722,8 @@ tm_status reconstruct_xo(const Solver& S, const void* xo, const void* be, const 
   const double rre = rr[0], rro = rr[1];
   *true_rel = bfull > 0.0 ? std::sqrt((rre + rro) / bfull) : 0.0;
   if (rr_odd) *rr_odd = rro;
-  if ((st = unpack_full_parity(lat, TM_F64, x, T, 0, 0, s)) != TM_OK) return st;
-  return unpack_full_parity(lat, TM_F64, x, W, 1, 0, s);
+  if ((st = unpack_full_parity(lat, TM_FX, x, T, 0, 0, s)) != TM_OK) return st;
+  return unpack_full_parity(lat, xo_prec, x, W, 1, 0, s);
 }
 
 tm_status launch_accumulate(const Solver& S, void* X, void* xs) {
@@ -971,10 +981,10 @@ static tm_status solve_one(tm_lattice lat, double* x, const double* b, const tm_
   Solver S{lat, s, P.flavour, 2.0 * lat->kappa * lat->mu, {0, 0, 0, 0}};
   for (int p = 0; p < 4; ++p) S.hb[p] = spinor_bytes_per_site(p) * lat->h;
   tm_status st = TM_OK;
-  // FP64 fields: 0 b_e, 1 b_o, 2 b', 3 X, 4 R, 5 P, 6 T, 7 W
+  // FP64 fields: 0 b_e, 1 b_o, 2 b', 3 X, 4 R, 5 P, 6 T, 7 W (room for the FX form each; T and W hold it)
   void* w[8];
   for (int k = 0; k < 8; ++k) {
-    w[k] = workspace(lat, k, S.hb[TM_F64], &st);
+    w[k] = workspace(lat, k, fx_field_bytes(lat->h), &st);
     if (st != TM_OK) return st;
   }
   void *be = w[0], *bo = w[1], *bp = w[2], *X = w[3], *R = w[4], *Pv = w[5], *T = w[6], *W = w[7];
@@ -1039,7 +1049,7 @@ static tm_status solve_one(tm_lattice lat, double* x, const double* b, const tm_
   if (reconstructed)
     st = TM_OK;
   else if (nr.xo_in_W)
-    st = reconstruct_xo(S, W, be, bo, bfull, x, T, R, Pv, &info->true_rel_residual);
+    st = reconstruct_xo(S, W, TM_FX, be, bo, bfull, x, T, R, Pv, &info->true_rel_residual);
   else
     st = reconstruct_check(S, X, be, bo, bfull, x, T, W, R, Pv, &info->true_rel_residual);
   if (st != TM_OK) return st;

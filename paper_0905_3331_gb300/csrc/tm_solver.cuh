@@ -32,7 +32,7 @@ tm_status prepare_source(const Solver& S, const double* b, void* be, void* bo, v
 // rr_odd (optional): ||(b - M x)_o||^2, the odd part of the full residual
 tm_status reconstruct_check(const Solver& S, const void* X, const void* be, const void* bo, double bfull, double* x,
                             void* T, void* W, void* R, void* Pv, double* true_rel, double* rr_odd = nullptr);
-tm_status reconstruct_xo(const Solver& S, const void* xo, const void* be, const void* bo, double bfull, double* x,
+tm_status reconstruct_xo(const Solver& S, const void* xo, int xo_prec, const void* be, const void* bo, double bfull, double* x,
                          void* T, void* R, void* Pv, double* true_rel, double* rr_odd = nullptr);
 tm_status launch_accumulate(const Solver& S, void* X, void* xs);  // X (FP64) += xs (FP32); xs = 0
 
@@ -40,7 +40,7 @@ struct NormalResult {
   int iters, updates;
   bool converged;
   double rr_true;   // ||bp - A X||^2, recomputed in FP64 (the iterated one when `pending`)
-  bool xo_in_W;     // W holds Qhat^{-f} X for the final X (left by the last FP64 residual)
+  bool xo_in_W;     // W holds Qhat^{-f} X for the final X in FX form (left by the last FP64 residual)
   bool pending;     // the last sloppy stage reached the tolerance; X is not yet confirmed in FP64
 };
 // With defer_final (mixed modes, FP64 updates), a sloppy stage that reaches the tolerance ends
