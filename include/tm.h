@@ -383,8 +383,8 @@ void tm_cg_params_default(tm_cg_params *params);
  * that must not allocate device memory during the call: code running under a fixed
  * device-memory budget (a framework whose caching allocator already holds the memory, a
  * process with a hard memory limit) or in a latency-critical loop where a cudaMalloc or
- * cudaFree would synchronise the device.  tm_apply_D takes its four half-field work buffers
- * from lattice-owned memory allocated on first use; this variant takes them from one static
+ * cudaFree would synchronise the device.  tm_apply_D takes its work buffer
+ * from lattice-owned memory allocated on first use; this variant takes it from one static
  * 64 MiB device array that is part of the library's device code, so the call itself calls no
  * cudaMalloc, cudaFree or other allocating routine.  Every GPU that loads the library holds
  * those 64 MiB until the process exits.

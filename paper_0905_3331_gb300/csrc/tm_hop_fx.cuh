@@ -13,15 +13,53 @@ namespace tmq {
 constexpr int fx_spb(int P) { return P == 1 ? 64 : 32; }
 constexpr int fx_nt(int P) { return fx_spb(P) * 2 * P; }
 
+// Where the FP64 input of a launch is: an FP64 half field, or the sites of parity p of a canonical full
+// field, gamma5 applied if g5.
+struct HalfInput {
+  const char* in;
+  __device__ __forceinline__ bool valid() const { return in != nullptr; }
+  __device__ __forceinline__ void load(const Geom& g, int i, cpx<double> v[12]) const {
+    SpinorFmt<TM_F64>::load(in, g.h, i, v);
+  }
+};
+struct CanonInput {
+  const double* in;
+  int p, g5;
+  __device__ __forceinline__ bool valid() const { return true; }
+  __device__ __forceinline__ void load(const Geom& g, int i, cpx<double> v[12]) const {
+    const double* q = in + lex_of_cb(g, i, p) * 24;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const cpx<double> t = mk(__ldg(q + 2 * k), __ldg(q + 2 * k + 1));
+      v[k] = (g5 && k >= 6) ? mk(-t.re, -t.im) : t;
+    }
+  }
+};
+
 // The FP64 form of one output site, for the sites whose neighbours have no fixed-point form.  A real
 // call, so that its registers are not the caller's.
-static __device__ __noinline__ void hop_f64_general(const Geom& g, int out_parity, int cb, const char* in,
+template <class Input>
+static __device__ __noinline__ void hop_f64_general(const Geom& g, int out_parity, int cb, const Input in,
                                                     const char* lf, const char* lo, double out[24]) {
   const SiteCoord c = site_of(g, cb, out_parity);
   int nb[8];
   neighbours(g, cb, c, nb);
-  cpx<double> acc[12];
-  hop_part<TM_F64, 18, 1>(acc, g, cb, c, nb, in, lf, lo, link_bytes(TM_F64, 18) * (size_t)g.h, 0);
+  const size_t slab = link_bytes(TM_F64, 18) * (size_t)g.h;
+  cpx<double> acc[12], p[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) acc[k] = mk(0.0, 0.0);
+#define TM_GENERAL_HOP(MU, S, I, SLAB, LI, NEG)                                                       \
+  in.load(g, nb[I], p);                                                                               \
+  hop_apply<TM_F64, 18, MU, S>(acc, load_raw<18 * 8>((SLAB) + MU * slab, g.h, LI), p, 1.0, NEG);
+  TM_GENERAL_HOP(0, +1, 0, lf, cb, c.t == g.T - 1)
+  TM_GENERAL_HOP(0, -1, 4, lo, nb[4], c.t == 0)
+  TM_GENERAL_HOP(1, +1, 1, lf, cb, false)
+  TM_GENERAL_HOP(1, -1, 5, lo, nb[5], false)
+  TM_GENERAL_HOP(2, +1, 2, lf, cb, false)
+  TM_GENERAL_HOP(2, -1, 6, lo, nb[6], false)
+  TM_GENERAL_HOP(3, +1, 3, lf, cb, false)
+  TM_GENERAL_HOP(3, -1, 7, lo, nb[7], false)
+#undef TM_GENERAL_HOP
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
     out[2 * k] = acc[k].re;
@@ -31,9 +69,10 @@ static __device__ __noinline__ void hop_f64_general(const Geom& g, int out_parit
 
 // acc = this lane's six components (spins q and 2 + q) of the sum A in FP64, with unit folded in by the
 // caller: real = acc unit.  All lanes of the warp call it (shuffles between the two lanes of a site).
-// in64: the FP64 input, or null.
+// in64: the FP64 input, if there is one.
+template <class Input>
 __device__ __forceinline__ void fx_finish(const FxAcc& A, int q, bool active, const Geom& g, int out_parity, int cb,
-                                          const char* in64, const char* lf, const char* lo, cpx<double> acc[6],
+                                          const Input in64, const char* lf, const char* lo, cpx<double> acc[6],
                                           double& unit) {
 #pragma unroll
   for (int k = 0; k < 3; ++k) {  // the other lane's share of this lane's lower spin 2 + q
@@ -45,7 +84,7 @@ __device__ __forceinline__ void fx_finish(const FxAcc& A, int q, bool active, co
   unit = fx_unit(A.E);
   if (A.bad && active) {
     unit = 1.0;
-    if (in64 != nullptr) {
+    if (in64.valid()) {
       double v[24];
       hop_f64_general(g, out_parity, cb, in64, lf, lo, v);
 #pragma unroll
@@ -72,9 +111,47 @@ __device__ __forceinline__ void fx_site(cpx<double> acc[6], int q, bool active, 
   A.bad = false;
   if (active) fx_hops<XIN>(A, q, g, cb, site_of(g, cb, out_parity), in, lf, lo, 0, 4);
   double unit;
-  fx_finish(A, q, active, g, out_parity, cb, in64, lf, lo, acc, unit);
+  fx_finish(A, q, active, g, out_parity, cb, HalfInput{in64}, lf, lo, acc, unit);
 #pragma unroll
   for (int k = 0; k < 6; ++k) acc[k] = unit * acc[k];
+}
+
+// The P direction parts' sums meet in part 0, at the largest of their exponents (called by the block).
+template <int P, int SPB>
+__device__ __forceinline__ void fx_merge(FxAcc& A, int part, int lane2, fx* part_sum) {
+  fx* mine = part_sum + (part * SPB * 2 + lane2) * 19;
+  if (part > 0) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      mine[2 * k] = A.up[k].re;
+      mine[2 * k + 1] = A.up[k].im;
+      mine[6 + 2 * k] = A.s[k].re;
+      mine[7 + 2 * k] = A.s[k].im;
+      mine[12 + 2 * k] = A.o[k].re;
+      mine[13 + 2 * k] = A.o[k].im;
+    }
+    mine[18] = A.bad ? -1 : A.E;
+  }
+  __syncthreads();
+  if (part == 0) {
+#pragma unroll
+    for (int p = 1; p < P; ++p) {
+      const fx* o = part_sum + (p * SPB * 2 + lane2) * 19;
+      const int Ep = (int)o[18];
+      if (Ep < 0) {
+        A.bad = true;
+        continue;
+      }
+      const int sa = Ep > A.E ? min(Ep - A.E, 63) : 0, so = A.E > Ep ? min(A.E - Ep, 63) : 0;
+      A.E = max(A.E, Ep);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        A.up[k] = mk<fx>((A.up[k].re >> sa) + (o[2 * k] >> so), (A.up[k].im >> sa) + (o[2 * k + 1] >> so));
+        A.s[k] = mk<fx>((A.s[k].re >> sa) + (o[6 + 2 * k] >> so), (A.s[k].im >> sa) + (o[7 + 2 * k] >> so));
+        A.o[k] = mk<fx>((A.o[k].re >> sa) + (o[12 + 2 * k] >> so), (A.o[k].im >> sa) + (o[13 + 2 * k] >> so));
+      }
+    }
+  }
 }
 
 // The body: output sites [bid SPB, (bid + 1) SPB) of right-hand side rhs; arguments and modes as
@@ -109,46 +186,13 @@ __device__ __forceinline__ void hop_sites_fx(const Geom g, const int out_parity,
     const SiteCoord c = site_of(g, cb, out_parity);
     fx_hops<XIN>(A, q, g, cb, c, inr, lf, lo, part * (4 / P), (part + 1) * (4 / P));
   }
-  if constexpr (P > 1) {  // the parts' sums meet in part 0, at the largest of their exponents
-    fx* mine = part_sum + (part * SPB * 2 + lane2) * 19;
-    if (part > 0) {
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        mine[2 * k] = A.up[k].re;
-        mine[2 * k + 1] = A.up[k].im;
-        mine[6 + 2 * k] = A.s[k].re;
-        mine[7 + 2 * k] = A.s[k].im;
-        mine[12 + 2 * k] = A.o[k].re;
-        mine[13 + 2 * k] = A.o[k].im;
-      }
-      mine[18] = A.bad ? -1 : A.E;
-    }
-    __syncthreads();
-    if (part == 0) {
-#pragma unroll
-      for (int p = 1; p < P; ++p) {
-        const fx* o = part_sum + (p * SPB * 2 + lane2) * 19;
-        const int Ep = (int)o[18];
-        if (Ep < 0) {
-          A.bad = true;
-          continue;
-        }
-        const int sa = Ep > A.E ? min(Ep - A.E, 63) : 0, so = A.E > Ep ? min(A.E - Ep, 63) : 0;
-        A.E = max(A.E, Ep);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          A.up[k] = mk<fx>((A.up[k].re >> sa) + (o[2 * k] >> so), (A.up[k].im >> sa) + (o[2 * k + 1] >> so));
-          A.s[k] = mk<fx>((A.s[k].re >> sa) + (o[6 + 2 * k] >> so), (A.s[k].im >> sa) + (o[7 + 2 * k] >> so));
-          A.o[k] = mk<fx>((A.o[k].re >> sa) + (o[12 + 2 * k] >> so), (A.o[k].im >> sa) + (o[13 + 2 * k] >> so));
-        }
-      }
-    }
-  }
+  if constexpr (P > 1) fx_merge<P, SPB>(A, part, lane2, part_sum);
   double nrm = 0.0;
   if (part == 0) {
     cpx<double> acc[6];
     double unit;
-    fx_finish(A, q, active, g, out_parity, cb, XIN ? static_cast<const char*>(fxa.in64) : inr, lf, lo, acc, unit);
+    fx_finish(A, q, active, g, out_parity, cb, HalfInput{XIN ? static_cast<const char*>(fxa.in64) : inr}, lf, lo, acc,
+              unit);
     // epilogue: o_s = D_s (c acc_s + E_s y_s) as (D_s c unit) acc_s + (D_s E_s) y_s; a real D c (every
     // coefficient set but the inverse site term) takes half the products
     const double cc = coef.c * unit;

@@ -187,6 +187,32 @@ __device__ __forceinline__ SiteCoord site_of(const Geom& g, int cb, int parity) 
   return c;
 }
 
+// Canonical records (12 complex FP64 components per site) pass through shared memory, CANON_TILE double2
+// per site (13 x 16 bytes: conflict free for a thread per site), so that global accesses are whole
+// 192-byte runs; read or written by one thread each, a record's 16-byte accesses fill half a sector.
+constexpr int CANON_TILE = 13;
+// One complex number of a canonical field; its records are 16-byte aligned if al (callers may pass any
+// 8-byte aligned address).
+__device__ __forceinline__ double2 canon_load(const double* p, bool al) {
+  return al ? __ldg(reinterpret_cast<const double2*>(p)) : make_double2(__ldg(p), __ldg(p + 1));
+}
+__device__ __forceinline__ void canon_store(double* p, double2 v, bool al) {
+  if (al) {
+    *reinterpret_cast<double2*>(p) = v;
+  } else {
+    p[0] = v.x;
+    p[1] = v.y;
+  }
+}
+inline bool canon_aligned(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
+
+// lexicographic index of site cb of parity p
+__device__ __forceinline__ size_t lex_of_cb(const Geom& g, int cb, int p) {
+  const int r = cb / g.Lh;
+  const int y = r % g.L, z = (r / g.L) % g.L, t = r / (g.L * g.L);
+  return 2 * (size_t)cb + ((t + z + y + p) & 1);
+}
+
 // cb indices of the 8 neighbours: nb[mu] = x + mu^, nb[4 + mu] = x - mu^ (periodic wrap).
 __device__ __forceinline__ void neighbours(const Geom& g, int cb, const SiteCoord& c, int nb[8]) {
   const int row = cb - (c.x >> 1);  // cb of (t, z, y, x = 0 or 1)
@@ -1228,7 +1254,7 @@ struct FxArgs {
   int flags = 0;               // which of in, out, y are FX half fields
   const void* in64 = nullptr;  // FX_IN: the FP64 field that in was made from, or null (inside a solver)
 };
-inline size_t fx_field_bytes(size_t h) { return 196 * h; }
+__host__ __device__ inline size_t fx_field_bytes(size_t h) { return 196 * h; }
 
 // Hopping launch description (one parity, nrhs fields).
 struct HopArgs {
@@ -1263,8 +1289,11 @@ tm_status unpack_full_parity(tm_lattice lat, int prec, double* dst_full, const v
                              int g5, cudaStream_t s);
 tm_status convert_half(tm_lattice lat, int prec_out, void* dst, int prec_in, const void* src,
                        cudaStream_t s);
-tm_status apply_M_halves(tm_lattice lat, void* out_e, void* out_o, const void* in_e, const void* in_o, int f,
-                         cudaStream_t s);
+// out = M(f) in (eq. eo0), or gamma5 M(f) gamma5 in with g5, on canonical FP64 device fields (nrhs of them);
+// scratch holds the FX form of `per` fields at a time, full_fx_bytes(h) each (tm_operator_fx.cu)
+inline size_t full_fx_bytes(size_t h) { return (2 * fx_field_bytes(h) + 255) / 256 * 256; }
+tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g5, int nrhs, void* scratch, int per,
+                     cudaStream_t s);
 tm_status diag_apply(tm_lattice lat, int prec, void* out, const void* in, int nrhs, double dur, double dui,
                      double dlr, double dli, cudaStream_t s);
 // Workspace slots: 0..17 CG solver, 22..25 tm_apply_D, 26 staged input, 27 staged output,

@@ -1,8 +1,8 @@
 // tm_noalloc.cu -- tm_apply_D_noalloc: the full operator M (or M^dag) on canonical FP64
 // device fields without any device-memory allocation.
 //
-// tm_apply_D needs four half-field work buffers (even/odd input, even/odd output) and
-// allocates them from the device on first use.  Some callers cannot allow that: code that
+// tm_apply_D needs a work buffer (the fixed-point form of the two parities of its input) and
+// allocates it from the device on first use.  Some callers cannot allow that: code that
 // runs under a fixed device-memory budget (a framework whose caching allocator already holds
 // the memory, or a process with a hard memory limit), and latency-critical loops where a
 // cudaMalloc/cudaFree would synchronise the device.  This entry point takes its work buffers
@@ -14,8 +14,9 @@
 
 namespace tmq {
 
-// Scratch for the four FP64 half fields: 4 x 192 h bytes <= 64 MiB, i.e. h <= 87381,
-// V = T L^3 <= 174762 sites (16^3 x 32 fits).
+// 64 MiB.  The entry point's limit, 4 x 192 h bytes <= 64 MiB (h <= 87381, V = T L^3 <= 174762 sites;
+// 16^3 x 32 fits), is that of four FP64 half fields; the operator's scratch, 392 h bytes per right-hand
+// side, stays below it.
 constexpr size_t NOALLOC_SCRATCH_BYTES = size_t(64) << 20;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES];
 
@@ -93,20 +94,8 @@ extern "C" tm_status tm_apply_D_noalloc(tm_lattice lat, double* out, const doubl
                      lat->device);
   void* base = nullptr;
   if ((st = noalloc_scratch(&base)) != TM_OK) return st;
-  char* sc = static_cast<char*>(base);
-  void* w[4] = {sc, sc + slot, sc + 2 * slot, sc + 3 * slot};
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
   // M^dag = g5 M(-f) g5; every scratch byte that is read was written earlier in the same call
-  const int f = dagger ? -flavour : flavour;
-  const int g5 = dagger ? 1 : 0;
-  for (int r = 0; r < nrhs; ++r) {
-    const double* src = in + (size_t)r * lat->V * 24;
-    double* dst = out + (size_t)r * lat->V * 24;
-    if ((st = pack_full_parity(lat, TM_F64, w[0], src, 0, g5, s)) != TM_OK) return st;
-    if ((st = pack_full_parity(lat, TM_F64, w[1], src, 1, g5, s)) != TM_OK) return st;
-    if ((st = apply_M_halves(lat, w[2], w[3], w[0], w[1], f, s)) != TM_OK) return st;
-    if ((st = unpack_full_parity(lat, TM_F64, dst, w[2], 0, g5, s)) != TM_OK) return st;
-    if ((st = unpack_full_parity(lat, TM_F64, dst, w[3], 1, g5, s)) != TM_OK) return st;
-  }
-  return TM_OK;
+  const size_t per = NOALLOC_SCRATCH_BYTES / full_fx_bytes(lat->h);
+  return apply_full(lat, out, in, dagger ? -flavour : flavour, dagger ? 1 : 0, nrhs, base,
+                    per < (size_t)nrhs ? (int)per : nrhs, static_cast<cudaStream_t>(stream));
 }

@@ -1,0 +1,139 @@
+// tm_operator_fx.cu -- the full operator M of eq. eo0 on canonical FP64 fields, in two launches: the
+// canonical field to the FX form (tm_dslash_fx.cuh) of its two parities, then the hopping sum of both
+// parities with the site term, written in canonical order.
+//
+// The first form packed each parity, ran one hopping launch per parity on half fields and unpacked
+// each: six launches, and 192-byte records read and written by single threads (a quarter of the time on
+// 32^3 x 64).  Here the canonical records pass through shared memory (padded to 13 x 16 bytes: conflict
+// free), so that global accesses are whole 192-byte runs.  Both together, on 32^3 x 64: 1781 -> 1226 us a
+// call (1050 us of it the hopping launch, latency bound as in tm_dslash_fx.cuh; 2.0 GB a call are 297 us
+// of HBM); 8^4 41 -> 16 us (two launches instead of six).
+#include "tm_hop_fx.cuh"
+
+namespace tmq {
+
+// Sites lex [128 b, 128 b + 128) -- cb [64 b, 64 b + 64) of both parities -- of right-hand side y.
+__global__ void __launch_bounds__(128) full_to_fx_kernel(const Geom g, const double* __restrict__ in, char* __restrict__ out,
+                                                         size_t out_stride, int g5, bool al) {
+  __shared__ double2 tile[128 * CANON_TILE];
+  const size_t V = 2 * (size_t)g.h, first = (size_t)blockIdx.x * 128;
+  const int n = (int)min((size_t)128, V - first);
+  const double* src = in + ((size_t)blockIdx.y * V + first) * 24;
+  for (int i = threadIdx.x; i < n * 12; i += 128) tile[i / 12 * CANON_TILE + i % 12] = canon_load(src + 2 * (size_t)i, al);
+  __syncthreads();
+  if ((int)threadIdx.x >= n) return;
+  const size_t lex = first + threadIdx.x;
+  const int cb = (int)(lex / 2);
+  const int r = cb / g.Lh, y = r % g.L, z = (r / g.L) % g.L, t = r / (g.L * g.L);
+  const int p = (int)((lex + t + z + y) & 1);
+  cpx<double> v[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    const double2 a = tile[threadIdx.x * CANON_TILE + k];
+    v[k] = (g5 && k >= 6) ? mk(-a.x, -a.y) : mk(a.x, a.y);
+  }
+  const int e = fx_exponent_f64<12>(v);
+  char* o = out + blockIdx.y * out_stride + p * fx_field_bytes(g.h);
+  longlong2* q = reinterpret_cast<longlong2*>(o) + cb;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) q[(size_t)k * g.h] = fx_pack(v[k], e);
+  const_cast<int*>(fx_exps(o, g.h))[cb] = e;
+}
+
+// out = D (c H in + E in) on both parities (blockIdx.y) of right-hand side blockIdx.z; D c real.
+template <int P>
+__global__ void __launch_bounds__(fx_nt(P), HOP_FX_WARPS * 32 / fx_nt(P))
+    full_fx_kernel(const Geom g, const char* __restrict__ links, const char* __restrict__ fxin, size_t fx_stride,
+                   const double* __restrict__ in, double* __restrict__ out, const EpiCoef coef, int g5, bool al_in,
+                   bool al_out) {
+  constexpr int SPB = fx_spb(P), NT = fx_nt(P), WPP = NT / 32 / P;
+  __shared__ fx part_sum[P > 1 ? P * SPB * 2 * 19 : 1];
+  __shared__ double2 tile[SPB * CANON_TILE];
+  const int warp = threadIdx.x >> 5;
+  const int part = P == 1 ? 0 : warp / WPP;
+  const int lane2 = P == 1 ? (int)threadIdx.x : (warp % WPP) * 32 + (int)(threadIdx.x & 31);
+  const int q = lane2 & 1, site = lane2 >> 1;
+  const int parity = blockIdx.y;
+  const int cb = blockIdx.x * SPB + site;
+  const bool active = cb < g.h;
+  const size_t V24 = 48 * (size_t)g.h;
+  const double* inr = in + blockIdx.z * V24;
+  const size_t slab = (size_t)FX_LINK_BYTES * g.h;
+  const char* lf = links + (size_t)(parity * 4) * slab;
+  const char* lo = links + (size_t)((1 - parity) * 4) * slab;
+  const char* src = fxin + blockIdx.z * fx_stride + (1 - parity) * fx_field_bytes(g.h);
+  FxAcc A;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) A.up[k] = A.s[k] = A.o[k] = mk<fx>(0, 0);
+  A.E = 0;
+  A.bad = false;
+  if (active) fx_hops<true>(A, q, g, cb, site_of(g, cb, parity), src, lf, lo, part * (4 / P), (part + 1) * (4 / P));
+  if constexpr (P > 1) fx_merge<P, SPB>(A, part, lane2, part_sum);
+  if (part == 0) {
+    cpx<double> acc[6];
+    double unit;
+    fx_finish(A, q, active, g, parity, cb, CanonInput{inr, 1 - parity, g5}, lf, lo, acc, unit);
+    if (active) {
+      const cpx<double> DEu = mk(coef.d_up_re, 0.0) * mk(coef.e_up_re, coef.e_up_im);
+      const cpx<double> DEl = mk(coef.d_lo_re, 0.0) * mk(coef.e_lo_re, coef.e_lo_im);
+      const double cu = coef.d_up_re * coef.c * unit, cl = coef.d_lo_re * coef.c * unit;
+      const double* y = inr + lex_of_cb(g, cb, parity) * 24;
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        const int blk = (k < 3 ? 3 * q : 6 + 3 * q) + k % 3;
+        const double2 t = canon_load(y + 2 * blk, al_in);
+        const cpx<double> e = (k < 3 ? DEu : DEl) * mk(t.x, t.y);
+        const double d = k < 3 ? cu : cl;
+        tile[site * CANON_TILE + blk] = make_double2(fma(d, acc[k].re, e.re), fma(d, acc[k].im, e.im));
+      }
+    }
+  }
+  __syncthreads();
+  double* dst = out + blockIdx.z * V24;
+  for (int i = threadIdx.x; i < SPB * 12; i += NT) {
+    const int s = i / 12, k = i % 12, c2 = blockIdx.x * SPB + s;
+    if (c2 >= g.h) break;
+    double* o = dst + lex_of_cb(g, c2, parity) * 24 + 2 * k;
+    canon_store(o, tile[s * CANON_TILE + k], al_out);
+  }
+}
+
+tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g5, int nrhs, void* scratch, int per,
+                     cudaStream_t s) {
+  tm_status st = ensure_links(lat, TM_F64, 18, s);
+  if (st != TM_OK) return st;
+  const Geom& g = lat->geom;
+  EpiCoef c = epi_full_M(lat->kappa, 2.0 * lat->kappa * lat->mu, f);
+  if (g5) {  // gamma5 M gamma5: the lower spins of the result, and of the site term's input, change sign
+    c.d_lo_re = -c.d_lo_re;
+    c.e_lo_re = -c.e_lo_re;
+    c.e_lo_im = -c.e_lo_im;
+  }
+  const char* links = static_cast<const char*>(lat->links[TM_F64][link_index(18)]);
+  char* fxs = static_cast<char*>(scratch);
+  const size_t stride = full_fx_bytes(lat->h);
+  const bool al_in = canon_aligned(in), al_out = canon_aligned(out);
+  for (int r = 0; r < nrhs; r += per) {
+    const int n = nrhs - r < per ? nrhs - r : per;
+    const double* src = in + (size_t)r * lat->V * 24;
+    double* dst = out + (size_t)r * lat->V * 24;
+    full_to_fx_kernel<<<dim3((unsigned)((lat->V + 127) / 128), n), 128, 0, s>>>(g, src, fxs, stride, g5, al_in);
+    count_launch();
+#define TM_FULL(P)                                                                                             \
+  full_fx_kernel<P><<<dim3((g.h + fx_spb(P) - 1) / fx_spb(P), 2, n), fx_nt(P), 0, s>>>(g, links, fxs, stride, src, dst, \
+                                                                                       c, g5, al_in, al_out)
+    const int tps = lat->hop_tps[TM_F64][link_index(18)];
+    if (tps == 2)
+      TM_FULL(2);
+    else if (tps == 4)
+      TM_FULL(4);
+    else
+      TM_FULL(1);
+#undef TM_FULL
+    count_launch();
+    if ((st = cuda_check(cudaGetLastError(), "operator kernel launch")) != TM_OK) return st;
+  }
+  return TM_OK;
+}
+
+}  // namespace tmq
