@@ -147,8 +147,8 @@ __device__ __forceinline__ fx fx_addsgn(fx a, fx x, int m) { return a + (x ^ (fx
 constexpr int FX_LINK_BYTES = 18 * 8;  // a link's 9 complex entries, words (re.lo, re.hi, im.lo, im.hi)
 
 // u = U h (S > 0) or U^dag h for a colour vector, h >> sh, in units of 2^(E - 1079)
-template <int S>
-__device__ __forceinline__ void fx_su3(const RawWords<FX_LINK_BYTES>& U, const cpx<fx> h[3], int sh, int one, cpx<fx> u[3]) {
+template <int S, class Link>
+__device__ __forceinline__ void fx_su3(Link U, const cpx<fx> h[3], int sh, int one, cpx<fx> u[3]) {
   FxLimbs hr[3], hi[3], hn[3];  // re, im, and -im (U h) or -re (U^dag h)
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -163,7 +163,8 @@ __device__ __forceinline__ void fx_su3(const RawWords<FX_LINK_BYTES>& U, const c
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
       const int k = S > 0 ? 3 * a + b : 3 * b + a;
-      const FxLimbs ur = {(int)U.w[4 * k + 1], (int)U.w[4 * k]}, ui = {(int)U.w[4 * k + 3], (int)U.w[4 * k + 2]};
+      const uint4 w = U(k);
+      const FxLimbs ur = {(int)w.y, (int)w.x}, ui = {(int)w.w, (int)w.z};
       const FxLimbs xr = S > 0 ? hn[b] : hi[b], xi = S > 0 ? hr[b] : hn[b];  // ui's partners
       if (b == 0) {
         p[0] = fx_mul(ur.hi, hr[b].hi);
@@ -199,26 +200,14 @@ struct FxAcc {
   bool bad;
 };
 
-// acc += one hop, from neighbour nbi and link (slab, li), of direction mu.  E grows to the neighbour's
-// exponent, acc is shifted right then.  Component q of (1 + S gamma_mu) v is v_q - S z v_partner for
-// q = 0 and v_1 - S sigma z v_partner for q = 1, z = 1 (t, y) or i (x, z), sigma = -1 for y and z
-// (sgn: the mask of sigma in this lane); the hop adds conj(-S sigma z) u to the partner's spin.
-template <bool XIN, int S>
-__device__ __forceinline__ void fx_hop(int mu, int q, int one, FxAcc& A, const char* in, int h, int nbi, const char* slab, int li,
-                                       bool negate) {
-  const RawWords<FX_LINK_BYTES> U = load_raw<FX_LINK_BYTES>(slab, h, li);
-  const bool tz = mu == 0 || mu == 3;
-  cpx<fx> v[6];
-  int e = fx_load<XIN>(in, h, nbi, 3 * q, tz ? 6 + 3 * q : 9 - 3 * q, v);
-  if (!XIN) {  // the site's exponent from the lane pair; both lanes keep the same E
-    const int eo = __shfl_xor_sync(__activemask(), e, 1);
-    if (eo > e) {
-      const int d = min(eo - e, 63);
-#pragma unroll
-      for (int k = 0; k < 6; ++k) v[k] = mk<fx>(v[k].re >> d, v[k].im >> d);
-      e = eo;
-    }
-  }
+// acc += one hop of direction mu: v the neighbour's component q and its partner, of exponent e, link(k) the
+// entry k of the hop's link.  E grows to the neighbour's exponent, acc is shifted right then.  Component
+// q of (1 + S gamma_mu) v is v_q - S z v_partner for q = 0 and v_1 - S sigma z v_partner for q = 1,
+// z = 1 (t, y) or i (x, z), sigma = -1 for y and z; the hop adds conj(-S sigma z) u to the partner's
+// spin.
+template <int S, class Link>
+__device__ __forceinline__ void fx_hop_apply(int mu, int q, int one, FxAcc& A, const cpx<fx> v[6], int e, Link link,
+                                             bool negate) {
   if (e >= A.E && e <= FX_EMAX && e != 0) {  // to e + 1: a later neighbour has to be twice as large to grow it again
     const int sh = min(e + 1 - A.E, 63);
 #pragma unroll
@@ -253,7 +242,7 @@ __device__ __forceinline__ void fx_hop(int mu, int q, int one, FxAcc& A, const c
     for (int c = 0; c < 3; ++c)
       hh[c] = mk<fx>(fx_addsgn(v[c].re, v[3 + c].im, ~m1), fx_addsgn(v[c].im, v[3 + c].re, m1));
   }
-  fx_su3<S>(U, hh, min(max(A.E - e, 0), 63), one, u);  // a zero or FX_BAD neighbour: any shift
+  fx_su3<S>(link, hh, min(max(A.E - e, 0), 63), one, u);  // a zero or FX_BAD neighbour: any shift
 #pragma unroll
   for (int a = 0; a < 3; ++a) A.up[a] = A.up[a] + u[a];
   if (mu == 0) {
@@ -272,6 +261,47 @@ __device__ __forceinline__ void fx_hop(int mu, int q, int one, FxAcc& A, const c
   }
 }
 
+// One hop read into registers and applied.
+template <bool XIN, int S>
+__device__ __forceinline__ void fx_hop(int mu, int q, int one, FxAcc& A, const char* in, int h, int nbi, const char* slab,
+                                       int li, bool negate) {
+  const RawWords<FX_LINK_BYTES> U = load_raw<FX_LINK_BYTES>(slab, h, li);
+  const bool tz = mu == 0 || mu == 3;
+  cpx<fx> v[6];
+  int e = fx_load<XIN>(in, h, nbi, 3 * q, tz ? 6 + 3 * q : 9 - 3 * q, v);
+  if (!XIN) {  // the site's exponent from the lane pair; both lanes keep the same E
+    const int eo = __shfl_xor_sync(__activemask(), e, 1);
+    if (eo > e) {
+      const int d = min(eo - e, 63);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) v[k] = mk<fx>(v[k].re >> d, v[k].im >> d);
+      e = eo;
+    }
+  }
+  fx_hop_apply<S>(mu, q, one, A, v, e,
+                  [&](int k) { return make_uint4(U.w[4 * k], U.w[4 * k + 1], U.w[4 * k + 2], U.w[4 * k + 3]); }, negate);
+}
+
+// The two neighbours of direction mu, and whether they lie across the lattice's edge.
+__device__ __forceinline__ void fx_neighbours(const Geom& g, int cb, const SiteCoord& c, int mu, int& nf, int& nb, bool& wf,
+                                              bool& wb) {
+  if (mu == 1) {
+    const int xp = c.x == g.L - 1 ? 0 : c.x + 1, xm = c.x == 0 ? g.L - 1 : c.x - 1;
+    const int row = cb - (c.x >> 1);
+    nf = row + (xp >> 1);
+    nb = row + (xm >> 1);
+    wf = wb = false;
+  } else {
+    const int co = mu == 0 ? c.t : (mu == 2 ? c.y : c.z);
+    const int ext = mu == 0 ? g.T : g.L;
+    const int st = mu == 0 ? g.st : (mu == 2 ? g.sy : g.sz);
+    wf = co == ext - 1;
+    wb = co == 0;
+    nf = wf ? cb - (ext - 1) * st : cb + st;
+    nb = wb ? cb + (ext - 1) * st : cb - st;
+  }
+}
+
 // The hops of directions [d0, d1) of a site in lane q, A in units of 2^(E - 1079).  The directions run
 // as one loop over the same code (what differs between them are signs and uniform branches): unrolled,
 // the sum was ~100 kB of instructions and the kernel waited for instruction fetch (16^3 x 32
@@ -284,23 +314,86 @@ __device__ __forceinline__ void fx_hops(FxAcc& A, int q, const Geom& g, int cb, 
 #pragma unroll 1
   for (int mu = d0; mu < d1; ++mu) {
     int nf, nb;
-    bool wf = false, wb = false;
-    if (mu == 1) {
-      const int xp = c.x == g.L - 1 ? 0 : c.x + 1, xm = c.x == 0 ? g.L - 1 : c.x - 1;
-      const int row = cb - (c.x >> 1);
-      nf = row + (xp >> 1);
-      nb = row + (xm >> 1);
-    } else {
-      const int co = mu == 0 ? c.t : (mu == 2 ? c.y : c.z);
-      const int ext = mu == 0 ? g.T : g.L;
-      const int st = mu == 0 ? g.st : (mu == 2 ? g.sy : g.sz);
-      wf = co == ext - 1;
-      wb = co == 0;
-      nf = wf ? cb - (ext - 1) * st : cb + st;
-      nb = wb ? cb + (ext - 1) * st : cb - st;
-    }
+    bool wf, wb;
+    fx_neighbours(g, cb, c, mu, nf, nb, wf, wb);
     fx_hop<XIN, +1>(mu, q, one, A, in, g.h, nf, lf + mu * slab, cb, mu == 0 && wf);
     fx_hop<XIN, -1>(mu, q, one, A, in, g.h, nb, lo + mu * slab, nb, mu == 0 && wb);
+  }
+}
+
+// The same for FX input with the next hop's neighbour and link copied to shared memory (cp.async) while
+// this hop is computed: in registers the two hops in flight would be 42 more of them.  For launches that
+// fill the chip (the full operator with one pair per site); the solvers' hopping launches on smaller
+// lattices lost 6 % with it (16^3 x 32, a CG of FP64 12.0 -> 12.7 ms), so they read into registers.
+// stage: FX_STAGE 16-byte slots per site and hop, slot k of the block's S sites at stage[k * S ..], two
+// hops.  Lane q's components are its own; lane 1 keeps them at site s ^ 4, so that the two lanes of four
+// sites (a shared-memory phase) use different banks.
+constexpr int FX_STAGE = 21;  // 9 link entries, 12 components
+__device__ __forceinline__ void fx_copy16(uint4* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+template <int SITES>
+__device__ __forceinline__ void fx_stage_hop(uint4* st, int site, int q, int h, const char* in, int nbi, const char* slab, int li,
+                                             int jb, int& e) {
+  const char* lp = slab + (size_t)li * 16;
+  const char* vp = in + (size_t)nbi * 16;
+  const size_t hb = (size_t)h * 16;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {  // link entries 0, 2, .. 8 by lane 0; 1, 3, 5, 7 by lane 1
+    const int n = 2 * k + q;
+    if (n < 9) fx_copy16(st + n * SITES + site, lp + n * hb);
+  }
+  uint4* const sv = st + (9 + 6 * q) * SITES + (site ^ (4 * q));
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    fx_copy16(sv + k * SITES, vp + (3 * q + k) * hb);
+    fx_copy16(sv + (3 + k) * SITES, vp + (jb + k) * hb);
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  e = __ldg(fx_exps(in, h) + nbi);
+}
+template <int SITES, int S>
+__device__ __forceinline__ void fx_apply_staged(const uint4* st, int site, int mu, int q, int one, FxAcc& A, int e, bool negate) {
+  cpx<fx> v[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const uint4 w = st[(9 + 6 * q + k) * SITES + (site ^ (4 * q))];
+    v[k] = mk<fx>((fx)(((unsigned long long)w.y << 32) | w.x), (fx)(((unsigned long long)w.w << 32) | w.z));
+  }
+  fx_hop_apply<S>(mu, q, one, A, v, e, [&](int k) { return st[k * SITES + site]; }, negate);
+}
+template <int SITES>
+__device__ __forceinline__ void fx_hops_staged(FxAcc& A, int q, const Geom& g, int cb, const SiteCoord& c, const char* in,
+                                               const char* lf, const char* lo, int d0, int d1, uint4* stage, int site) {
+  const size_t slab = (size_t)FX_LINK_BYTES * g.h;
+  const int one = fx_one();
+  uint4* const s1 = stage + FX_STAGE * SITES;
+  const unsigned mask = __activemask();
+  int nf, nb, e0, e1 = 0;
+  bool wf, wb;
+  fx_neighbours(g, cb, c, d0, nf, nb, wf, wb);
+  fx_stage_hop<SITES>(stage, site, q, g.h, in, nf, lf + d0 * slab, cb, (d0 == 0 || d0 == 3) ? 6 + 3 * q : 9 - 3 * q, e0);
+#pragma unroll 1
+  for (int mu = d0; mu < d1; ++mu) {
+    const int jb = (mu == 0 || mu == 3) ? 6 + 3 * q : 9 - 3 * q;
+    fx_stage_hop<SITES>(s1, site, q, g.h, in, nb, lo + mu * slab, nb, jb, e1);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncwarp(mask);
+    fx_apply_staged<SITES, +1>(stage, site, mu, q, one, A, e0, mu == 0 && wf);
+    __syncwarp(mask);
+    const bool wrap = mu == 0 && wb;
+    if (mu + 1 < d1) {
+      fx_neighbours(g, cb, c, mu + 1, nf, nb, wf, wb);
+      fx_stage_hop<SITES>(stage, site, q, g.h, in, nf, lf + (mu + 1) * slab, cb,
+                          (mu + 1 == 3) ? 6 + 3 * q : 9 - 3 * q, e0);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncwarp(mask);
+    fx_apply_staged<SITES, -1>(s1, site, mu, q, one, A, e1, wrap);
+    __syncwarp(mask);
   }
 }
 

@@ -6,8 +6,14 @@
 // each: six launches, and 192-byte records read and written by single threads (a quarter of the time on
 // 32^3 x 64).  Here the canonical records pass through shared memory (padded to 13 x 16 bytes: conflict
 // free), so that global accesses are whole 192-byte runs.  Both together, on 32^3 x 64: 1781 -> 1226 us a
-// call (1050 us of it the hopping launch, latency bound as in tm_dslash_fx.cuh; 2.0 GB a call are 297 us
-// of HBM); 8^4 41 -> 16 us (two launches instead of six).
+// call (most of it the hopping launch, latency bound as in tm_dslash_fx.cuh; 2.0 GB a call are 297 us of
+// HBM); 8^4 41 -> 16 us (two launches instead of six).
+//
+// One thread pair per site takes the next hop's neighbour and link into shared memory (cp.async) while it
+// computes this one (fx_hops_staged): 32^3 x 64 1226 -> 1124 us, two fields of 20 x 14^3 79.9 -> 77.7.
+// Several pairs per site (small lattices) read into registers: they have more hops in flight as it is,
+// and staging cost 3 % there.  Both are programmatic dependent launches: the second's blocks are resident
+// when the first's last ones end.
 #include "tm_hop_fx.cuh"
 
 namespace tmq {
@@ -19,6 +25,8 @@ __global__ void __launch_bounds__(128) full_to_fx_kernel(const Geom g, const dou
   const size_t V = 2 * (size_t)g.h, first = (size_t)blockIdx.x * 128;
   const int n = (int)min((size_t)128, V - first);
   const double* src = in + ((size_t)blockIdx.y * V + first) * 24;
+  pdl_wait();
+  pdl_allow();
   for (int i = threadIdx.x; i < n * 12; i += 128) tile[i / 12 * CANON_TILE + i % 12] = canon_load(src + 2 * (size_t)i, al);
   __syncthreads();
   if ((int)threadIdx.x >= n) return;
@@ -47,8 +55,13 @@ __global__ void __launch_bounds__(fx_nt(P), HOP_FX_WARPS * 32 / fx_nt(P))
                    const double* __restrict__ in, double* __restrict__ out, const EpiCoef coef, int g5, bool al_in,
                    bool al_out) {
   constexpr int SPB = fx_spb(P), NT = fx_nt(P), WPP = NT / 32 / P;
-  __shared__ fx part_sum[P > 1 ? P * SPB * 2 * 19 : 1];
-  __shared__ double2 tile[SPB * CANON_TILE];
+  constexpr bool STAGED = P == 1;
+  constexpr int TILE = SPB * CANON_TILE * 16, SUMS = P > 1 ? P * SPB * 2 * 19 * 8 : 0;
+  constexpr int STAGE = STAGED ? SPB * 2 * FX_STAGE * 16 : 0;
+  constexpr int SMEM = STAGE > TILE ? STAGE : (SUMS > TILE ? SUMS : TILE);
+  // the staged hops or the parts' sums, then the results
+  __shared__ __align__(16) char smem[SMEM];
+  double2* const tile = reinterpret_cast<double2*>(smem);
   const int warp = threadIdx.x >> 5;
   const int part = P == 1 ? 0 : warp / WPP;
   const int lane2 = P == 1 ? (int)threadIdx.x : (warp % WPP) * 32 + (int)(threadIdx.x & 31);
@@ -67,8 +80,17 @@ __global__ void __launch_bounds__(fx_nt(P), HOP_FX_WARPS * 32 / fx_nt(P))
   for (int k = 0; k < 3; ++k) A.up[k] = A.s[k] = A.o[k] = mk<fx>(0, 0);
   A.E = 0;
   A.bad = false;
-  if (active) fx_hops<true>(A, q, g, cb, site_of(g, cb, parity), src, lf, lo, part * (4 / P), (part + 1) * (4 / P));
-  if constexpr (P > 1) fx_merge<P, SPB>(A, part, lane2, part_sum);
+  pdl_wait();
+  pdl_allow();
+  if (active) {
+    const SiteCoord c = site_of(g, cb, parity);
+    if constexpr (STAGED)
+      fx_hops_staged<SPB>(A, q, g, cb, c, src, lf, lo, 0, 4, reinterpret_cast<uint4*>(smem), lane2 >> 1);
+    else
+      fx_hops<true>(A, q, g, cb, c, src, lf, lo, part * (4 / P), (part + 1) * (4 / P));
+  }
+  if constexpr (P > 1) fx_merge<P, SPB>(A, part, lane2, reinterpret_cast<fx*>(smem));
+  __syncthreads();
   if (part == 0) {
     cpx<double> acc[6];
     double unit;
@@ -117,11 +139,13 @@ tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g
     const int n = nrhs - r < per ? nrhs - r : per;
     const double* src = in + (size_t)r * lat->V * 24;
     double* dst = out + (size_t)r * lat->V * 24;
-    full_to_fx_kernel<<<dim3((unsigned)((lat->V + 127) / 128), n), 128, 0, s>>>(g, src, fxs, stride, g5, al_in);
+    cudaError_t e =
+        launch_pdl(full_to_fx_kernel, dim3((unsigned)((lat->V + 127) / 128), n), dim3(128), s, g, src, fxs, stride, g5, al_in);
+    if ((st = cuda_check(e, "operator kernel launch")) != TM_OK) return st;
     count_launch();
-#define TM_FULL(P)                                                                                             \
-  full_fx_kernel<P><<<dim3((g.h + fx_spb(P) - 1) / fx_spb(P), 2, n), fx_nt(P), 0, s>>>(g, links, fxs, stride, src, dst, \
-                                                                                       c, g5, al_in, al_out)
+#define TM_FULL(P)                                                                                                \
+  e = launch_pdl(full_fx_kernel<P>, dim3((g.h + fx_spb(P) - 1) / fx_spb(P), 2, n), dim3(fx_nt(P)), s, g, links,  \
+                 fxs, stride, src, dst, c, g5, al_in, al_out)
     const int tps = lat->hop_tps[TM_F64][link_index(18)];
     if (tps == 2)
       TM_FULL(2);
@@ -131,7 +155,8 @@ tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g
       TM_FULL(1);
 #undef TM_FULL
     count_launch();
-    if ((st = cuda_check(cudaGetLastError(), "operator kernel launch")) != TM_OK) return st;
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if ((st = cuda_check(e, "operator kernel launch")) != TM_OK) return st;
   }
   return TM_OK;
 }
