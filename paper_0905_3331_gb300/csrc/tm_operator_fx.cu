@@ -12,8 +12,7 @@
 // One thread pair per site takes the next hop's neighbour and link into shared memory (cp.async) while it
 // computes this one (fx_hops_staged): 32^3 x 64 1226 -> 1124 us, two fields of 20 x 14^3 79.9 -> 77.7.
 // Several pairs per site (small lattices) read into registers: they have more hops in flight as it is,
-// and staging cost 3 % there.  Both are programmatic dependent launches: the second's blocks are resident
-// when the first's last ones end.
+// and staging cost 3 % there.
 #include "tm_hop_fx.cuh"
 
 namespace tmq {
@@ -25,8 +24,6 @@ __global__ void __launch_bounds__(128) full_to_fx_kernel(const Geom g, const dou
   const size_t V = 2 * (size_t)g.h, first = (size_t)blockIdx.x * 128;
   const int n = (int)min((size_t)128, V - first);
   const double* src = in + ((size_t)blockIdx.y * V + first) * 24;
-  pdl_wait();
-  pdl_allow();
   for (int i = threadIdx.x; i < n * 12; i += 128) tile[i / 12 * CANON_TILE + i % 12] = canon_load(src + 2 * (size_t)i, al);
   __syncthreads();
   if ((int)threadIdx.x >= n) return;
@@ -80,8 +77,6 @@ __global__ void __launch_bounds__(fx_nt(P), HOP_FX_WARPS * 32 / fx_nt(P))
   for (int k = 0; k < 3; ++k) A.up[k] = A.s[k] = A.o[k] = mk<fx>(0, 0);
   A.E = 0;
   A.bad = false;
-  pdl_wait();
-  pdl_allow();
   if (active) {
     const SiteCoord c = site_of(g, cb, parity);
     if constexpr (STAGED)
@@ -139,13 +134,11 @@ tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g
     const int n = nrhs - r < per ? nrhs - r : per;
     const double* src = in + (size_t)r * lat->V * 24;
     double* dst = out + (size_t)r * lat->V * 24;
-    cudaError_t e =
-        launch_pdl(full_to_fx_kernel, dim3((unsigned)((lat->V + 127) / 128), n), dim3(128), s, g, src, fxs, stride, g5, al_in);
-    if ((st = cuda_check(e, "operator kernel launch")) != TM_OK) return st;
+    full_to_fx_kernel<<<dim3((unsigned)((lat->V + 127) / 128), n), 128, 0, s>>>(g, src, fxs, stride, g5, al_in);
     count_launch();
-#define TM_FULL(P)                                                                                                \
-  e = launch_pdl(full_fx_kernel<P>, dim3((g.h + fx_spb(P) - 1) / fx_spb(P), 2, n), dim3(fx_nt(P)), s, g, links,  \
-                 fxs, stride, src, dst, c, g5, al_in, al_out)
+#define TM_FULL(P)                                                                                             \
+  full_fx_kernel<P><<<dim3((g.h + fx_spb(P) - 1) / fx_spb(P), 2, n), fx_nt(P), 0, s>>>(g, links, fxs, stride, src, dst, \
+                                                                                       c, g5, al_in, al_out)
     const int tps = lat->hop_tps[TM_F64][link_index(18)];
     if (tps == 2)
       TM_FULL(2);
@@ -155,8 +148,7 @@ tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g
       TM_FULL(1);
 #undef TM_FULL
     count_launch();
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if ((st = cuda_check(e, "operator kernel launch")) != TM_OK) return st;
+    if ((st = cuda_check(cudaGetLastError(), "operator kernel launch")) != TM_OK) return st;
   }
   return TM_OK;
 }
