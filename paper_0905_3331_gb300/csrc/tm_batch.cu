@@ -90,18 +90,23 @@ __global__ void plans_init_kernel(Plans L) {
 // storage; serv = 1: the FP64 service of stopped systems, where K4's residual update uses alpha = 1
 // (r = b' - A X from r = b') and the reduction stores ||r||^2 in B.result.  A system that stopped
 // since the list was built (a breakdown in K2) is skipped.
+// FP32 / FP16 storage with one thread per site: 20 warps per SM (96 registers).  The launches wait for
+// loads (12 systems on 16^3 x 32, FP32/12: long scoreboard 6.2 of 10.3 cycles an issue at 20 warps, issue
+// slots 47 % busy, DRAM 35 %); with 16 warps of 128 registers the twelve solves took 66.7 ms, with 20
+// 63.5, with 24 (80 registers, spilled) 63.4.
 constexpr int hop_batch_nt(int prec, int tps) { return prec == TM_F64 ? fx_nt(1) : hop_spb(tps) * tps; }
 constexpr int hop_batch_min_blocks(int prec, int nreal, int tps) {
-  return prec == TM_F64 ? 16 * 32 / fx_nt(1) : (tps == 1 && (prec == TM_F32 || prec == TM_F16)) ? 512 / hop_spb(1) : 1;  // 8 blocks of 64 (128 registers)
+  return prec == TM_F64 ? 16 * 32 / fx_nt(1) : (tps == 1 && (prec == TM_F32 || prec == TM_F16)) ? 640 / hop_spb(1) : 1;
 }
 
 template <int PREC, int NREAL, bool HAS_Y, int MODE, int TPS>
 __global__ void __launch_bounds__(hop_batch_nt(PREC, TPS), hop_batch_min_blocks(PREC, NREAL, TPS))
     hop_batch_kernel(const BatchSys* __restrict__ systems, const CGState* __restrict__ states, Plan plan, int serv,
-                     int in_sel, int y_sel, int out_sel, int kk, int out_parity) {
+                     int in_sel, int y_sel, int out_sel, int kk, int out_parity, const int* loops) {
   const int total = plan.start[plan.nlat];
+  const bool rev = plan_reversed(loops, kk);
   for (int v = blockIdx.x; v < total; v += gridDim.x) {
-    const int2 m = plan_item(plan, v);
+    const int2 m = plan_item(plan, rev ? total - 1 - v : v);
     const CGState& S = states[m.x];
     if (serv ? !(S.done && !S.finished) : S.done) continue;  // block-uniform
     const BatchSys& B = systems[m.x];
@@ -129,8 +134,9 @@ __global__ void __launch_bounds__(BNT) cg_update_batch_kernel(const BatchSys* __
                                                               cudaGraphConditionalHandle cond_serv, int use_cond) {
   typedef typename SpinorFmt<PP>::real RP;
   const int total = L.upd.start[L.upd.nlat];
+  const bool rev = plan_reversed(&gl->loops, 4);
   for (int v = blockIdx.x; v < total; v += gridDim.x) {
-    const int2 m = plan_item(L.upd, v);
+    const int2 m = plan_item(L.upd, rev ? total - 1 - v : v);
     const BatchSys& B = systems[m.x];
     CGState& S = L.states[m.x];
     const int iter = S.iter;
@@ -295,13 +301,13 @@ __global__ void __launch_bounds__(BNT) serv_convert_kernel(const BatchSys* __res
 template <int PREC, int NREAL, int TPS>
 static tm_status launch_hop_batch(const BatchSys* d_sys, const CGState* d_st, const Plan& plan, int cap, int serv,
                                   int in_sel, int y_sel, int out_sel, int kk, int parity, int mode, bool has_y,
-                                  cudaStream_t s) {
+                                  const int* loops, cudaStream_t s) {
   constexpr int NT = hop_batch_nt(PREC, TPS);
 #define TM_GL(HY, MD)                                                                                  \
   {                                                                                                    \
     auto kern = hop_batch_kernel<PREC, NREAL, HY, MD, TPS>;                                            \
     kern<<<resident_grid(kern, NT, cap), NT, 0, s>>>(d_sys, d_st, plan, serv, in_sel, y_sel, out_sel, kk, \
-                                                     parity);                                          \
+                                                     parity, loops);                                   \
   }
   if (!has_y && mode == 0)
     TM_GL(false, 0)
@@ -328,20 +334,21 @@ struct BatchLaunch {
   int K;                    // systems per thread
   const BatchGroup* grp;    // the groups (K > 1)
   Plan gplan;               // their work list
+  const int* loops;         // iterations so far (plan_reversed), or nullptr
 };
 
 static tm_status hop_batch(const BatchLaunch& L, int in_sel, int y_sel, int out_sel, int kk, int parity, int mode,
                            bool has_y, cudaStream_t s) {
   if (L.K > 1)
     return launch_hop_group(L.prec, L.nreal, L.K, L.sys, L.grp, L.st, L.gplan, L.cap, in_sel, y_sel, out_sel, kk,
-                            parity, mode, has_y, s);
+                            parity, mode, has_y, L.loops, s);
   if (L.prec == TM_F64)
     return launch_hop_batch<TM_F64, 18, 1>(L.sys, L.st, L.plan, L.cap, L.serv, in_sel, y_sel, out_sel, kk, parity, mode,
-                                           has_y, s);
+                                           has_y, L.loops, s);
 #define TM_B(P, N, T)                                                                                      \
   if (L.prec == P && L.nreal == N && L.tps == T)                                                          \
     return launch_hop_batch<P, N, T>(L.sys, L.st, L.plan, L.cap, L.serv, in_sel, y_sel, out_sel, kk, parity, mode, \
-                                     has_y, s);
+                                     has_y, L.loops, s);
 #define TM_BT(P, N) TM_B(P, N, 1) TM_B(P, N, 2) TM_B(P, N, 4)
   TM_BT(TM_F32, 18) TM_BT(TM_F32, 12) TM_BT(TM_F32, 8) TM_BT(TM_F16, 18) TM_BT(TM_F16, 12) TM_BT(TM_F16, 8)
 #undef TM_BT
@@ -745,8 +752,8 @@ extern "C" tm_status tm_solve_cg_batch(const tm_system* systems, int nsys, const
     Y.hat(4, li) = (int)((lats[li].lat->h + hop_spb(1) - 1) / hop_spb(1));
   }
   const Plans plans = Y.plans();
-  BatchLaunch GL{sp, sl, 1, 0, d_sys, plans.states, plans.hop, npart, 1, Y.groups, plans.ghop};
-  BatchLaunch GD{TM_F64, 18, 1, 1, d_sys64, plans.states, plans.shop, npart, 1, nullptr, plans.ghop};
+  BatchLaunch GL{sp, sl, 1, 0, d_sys, plans.states, plans.hop, npart, 1, Y.groups, plans.ghop, nullptr};
+  BatchLaunch GD{TM_F64, 18, 1, 1, d_sys64, plans.states, plans.shop, npart, 1, nullptr, plans.ghop, nullptr};
   CGState* d_st = reinterpret_cast<CGState*>(base + off_state);
   BatchGlobal* d_gl = reinterpret_cast<BatchGlobal*>(base + off_gl);
   double* d_part = reinterpret_cast<double*>(base + off_part);
@@ -851,6 +858,7 @@ extern "C" tm_status tm_solve_cg_batch(const tm_system* systems, int nsys, const
     hgl = BatchGlobal{unfinished, 0, P.max_iter + 16, 0u, nsys, 0, delta2, SLOPPY_GROWTH * SLOPPY_GROWTH};
     st = cuda_check(cudaMemcpyAsync(d_st, hst.data(), sizeof(CGState) * nsys, cudaMemcpyHostToDevice, s), "state");
     if (st == TM_OK) st = cuda_check(cudaMemcpyAsync(d_gl, &hgl, sizeof(hgl), cudaMemcpyHostToDevice, s), "state");
+    GL.loops = &d_gl->loops;
     if (st == TM_OK) {
       plans_init_kernel<<<1, 32 * NPLANS, 0, s>>>(plans);
       count_launch();

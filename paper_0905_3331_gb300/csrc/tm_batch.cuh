@@ -68,6 +68,15 @@ struct Plans {
   const BatchGroup* groups;   // [ngroups] the groups, lattice by lattice
 };
 
+// The direction of a launch over its work list, alternating from launch to launch: k-th launch of the
+// iteration *loops (5 launches each; nullptr: 0).  A batch's vectors are several times the L2 (twelve
+// systems on 16^3 x 32: 75 MB a vector), so a launch that starts where the one before it started finds
+// nothing of what that one wrote; starting where it ended, it finds the last ~100 MB.
+// (those twelve solves: 68.1 -> 66.7 ms).
+__device__ __forceinline__ bool plan_reversed(const int* loops, int k) {
+  return ((k + (loops != nullptr ? *loops : 0)) & 1) != 0;
+}
+
 __device__ __forceinline__ int2 plan_item(const Plan& P, int v) {
   int li = 0;
   while (li + 1 < P.nlat && v >= P.start[li + 1]) ++li;
@@ -80,7 +89,7 @@ __device__ __forceinline__ int2 plan_item(const Plan& P, int v) {
 // (tm_batch_group.cu): FP32 or FP16 storage, HOP_NT sites per block.
 tm_status launch_hop_group(int prec, int nreal, int K, const BatchSys* d_sys, const BatchGroup* d_grp,
                            const CGState* d_st, const Plan& plan, int cap, int in_sel, int y_sel, int out_sel, int kk,
-                           int parity, int mode, bool has_y, cudaStream_t s);
+                           int parity, int mode, bool has_y, const int* loops, cudaStream_t s);
 
 // Blocks of a launch: as many as the GPU keeps resident (at most `cap`, the blocks of a full list).
 template <class Kern>

@@ -127,23 +127,23 @@ template <int PREC, int NREAL, bool HAS_Y, int MODE, int K>
 __global__ void __launch_bounds__(HOP_NT, K == 2 ? 3 : 2)
     hop_group_kernel(const BatchSys* __restrict__ systems, const BatchGroup* __restrict__ groups,
                      const CGState* __restrict__ states, Plan plan, int in_sel, int y_sel, int out_sel, int kk,
-                     int out_parity) {
+                     int out_parity, const int* loops) {
   __shared__ double sh[HOP_NT / 32];
   const int total = plan.start[plan.nlat];
+  const bool rev = plan_reversed(loops, kk);
   for (int v = blockIdx.x; v < total; v += gridDim.x)
-    group_block<PREC, NREAL, HAS_Y, MODE, K>(systems, groups, states, plan_item(plan, v), in_sel, y_sel, out_sel, kk,
-                                             out_parity, sh);
+    group_block<PREC, NREAL, HAS_Y, MODE, K>(systems, groups, states, plan_item(plan, rev ? total - 1 - v : v), in_sel, y_sel, out_sel, kk, out_parity, sh);
 }
 
 template <int PREC, int NREAL, int K>
 static tm_status launch_t(const BatchSys* d_sys, const BatchGroup* d_grp, const CGState* d_st, const Plan& plan,
                           int cap, int in_sel, int y_sel, int out_sel, int kk, int parity, int mode, bool has_y,
-                          cudaStream_t s) {
+                          const int* loops, cudaStream_t s) {
 #define TM_GL(HY, MD)                                                                                   \
   {                                                                                                     \
     auto kern = hop_group_kernel<PREC, NREAL, HY, MD, K>;                                               \
     kern<<<resident_grid(kern, HOP_NT, cap), HOP_NT, 0, s>>>(d_sys, d_grp, d_st, plan, in_sel, y_sel, out_sel, \
-                                                             kk, parity);                              \
+                                                             kk, parity, loops);                       \
   }
   if (!has_y && mode == 0)
     TM_GL(false, 0)
@@ -160,10 +160,10 @@ static tm_status launch_t(const BatchSys* d_sys, const BatchGroup* d_grp, const 
 
 tm_status launch_hop_group(int prec, int nreal, int K, const BatchSys* d_sys, const BatchGroup* d_grp,
                            const CGState* d_st, const Plan& plan, int cap, int in_sel, int y_sel, int out_sel, int kk,
-                           int parity, int mode, bool has_y, cudaStream_t s) {
+                           int parity, int mode, bool has_y, const int* loops, cudaStream_t s) {
 #define TM_B(P, N, KK)                                                                                          \
   if (prec == P && nreal == N && K == KK)                                                                       \
-    return launch_t<P, N, KK>(d_sys, d_grp, d_st, plan, cap, in_sel, y_sel, out_sel, kk, parity, mode, has_y, s);
+    return launch_t<P, N, KK>(d_sys, d_grp, d_st, plan, cap, in_sel, y_sel, out_sel, kk, parity, mode, has_y, loops, s);
 #define TM_BK(P, N) TM_B(P, N, 2) TM_B(P, N, 4)
   TM_BK(TM_F32, 18) TM_BK(TM_F32, 12) TM_BK(TM_F32, 8) TM_BK(TM_F16, 18) TM_BK(TM_F16, 12) TM_BK(TM_F16, 8)
 #undef TM_BK
