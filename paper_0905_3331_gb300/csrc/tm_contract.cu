@@ -44,7 +44,7 @@ constexpr int C_ROWG = 22;             // row groups of 8: 176 operand rows
 constexpr int C_LBO = C_ROWG * 128;    // bytes between k groups; 128 between row groups
 constexpr int C_RED = 4 * 24 * 24 * 3 * 8;  // the drained sums, in the operand tile's place
 constexpr int C_OPER = CT / 8 * C_LBO > C_RED ? CT / 8 * C_LBO : C_RED;
-constexpr int C_ROWP = CT * 16 + 64;   // bytes per propagator of a raw tile (padded: conflict-free reads)
+constexpr int C_ROWP = CT * 16 + 32;   // bytes per propagator of a raw tile (padded: conflict-free reads)
 constexpr int C_RAW = 12 * C_ROWP;
 constexpr int C_SMEM = C_OPER + 2 * C_RAW;
 constexpr int C_COLS = 256;            // TMEM columns per block
@@ -95,8 +95,8 @@ __device__ __forceinline__ bool c_wait(unsigned bar, unsigned parity) {
   return false;
 }
 
-// The FP64 number with words (lo, hi) as an integer of exponent E, v 2^(E - 1077), rounded, with 128
-// added to each of its seven balanced digits
+// |x| as an integer of exponent E, v 2^(E - 1077), rounded, with 128 added to each of its seven balanced
+// digits
 __device__ __forceinline__ unsigned long long c_digits(double x, int E) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int sh = E - (int)((hi >> 20) & 0x7ffu);  // >= 1; zero and denormal reals are shifted out
@@ -104,11 +104,11 @@ __device__ __forceinline__ unsigned long long c_digits(double x, int E) {
       ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 35) | ((unsigned long long)lo << 3);
   unsigned long long q;
   asm("shr.u64 %0, %1, %2;" : "=l"(q) : "l"(w), "r"(sh));  // PTX clamps shifts above 63: 0
-  const long long s = (long long)((int)hi >> 31);
-  return (unsigned long long)(((long long)q ^ s) + (2 * 0x80808080808080ll + 1) + (long long)(hi >> 31)) >> 1;
+  return (q + (2 * 0x80808080808080ull + 1)) >> 1;
 }
 
-// Eight reals of one operand row: the seven digit rows' 16 bytes each
+// Eight reals of one operand row: the seven digit rows' 16 bytes each.  The digits of |x| take x's sign in
+// the fp16 operation that removes their offset.
 __device__ __forceinline__ void c_store_row(char* tile, int row, const double x[8], int E) {
   unsigned d[7][4];  // digit i: components 2 m, 2 m + 1 in word m
   const __half2 off = __half2half2(__ushort_as_half(0xe480));  // -1152
@@ -116,12 +116,14 @@ __device__ __forceinline__ void c_store_row(char* tile, int row, const double x[
   for (int m = 0; m < 4; ++m) {
     const unsigned long long a = c_digits(x[2 * m], E), b = c_digits(x[2 * m + 1], E);
     const unsigned w[2][2] = {{(unsigned)a, (unsigned)b}, {(unsigned)(a >> 32), (unsigned)(b >> 32)}};
+    const unsigned sb = (__byte_perm(__double2hiint(x[2 * m]), __double2hiint(x[2 * m + 1]), 0x7632) & 0x80008000u) | 0x3c003c00u;
+    const __half2 sgn = *reinterpret_cast<const __half2*>(&sb), soff = __hmul2(sgn, off);  // +-1, -+1152
 #pragma unroll
     for (int byte = 0; byte < 7; ++byte) {
       // bytes (a.b, b.b) of two digits, then 0x64 above each: the halves 1024 + digit + 128
       const unsigned g = __byte_perm(w[byte / 4][0], w[byte / 4][1], (byte & 2) ? 0x7362 : 0x5140);
       const unsigned h = __byte_perm(g, 0x64646464u, (byte & 1) ? 0x4342 : 0x4140);
-      const __half2 v = __hadd2(*reinterpret_cast<const __half2*>(&h), off);
+      const __half2 v = __hfma2(*reinterpret_cast<const __half2*>(&h), sgn, soff);
       d[6 - byte][m] = *reinterpret_cast<const unsigned*>(&v);
     }
   }
@@ -137,13 +139,15 @@ __device__ __forceinline__ void c_mad(long long& s, int a, int b) {
 }
 
 // partial[t][bx][pair] (complex): block bx of timeslice t sums its tiles of components.
-// 24^3 x 48: 5.53 -> 0.77 ms (1.53 GB: 225 us of HBM).  Bound by the latency of a tile's steps between its
-// two block barriers (issue 36% active with two blocks per SM; the tensor core 15%): without the
-// conversion 0.55 ms, without the drains 0.68 ms.
+// 24^3 x 48: 5.53 -> 0.72 ms (1.53 GB: 225 us of HBM).  With two barriers per tile, the next tile read after
+// them, it was 0.77; conflict-free raw rows and the sign taken in fp16 (an eighth of the instructions)
+// brought 0.05.  Bound by the latency of a block's steps, which the other resident block covers in part:
+// issue 43% active, ALU 45%, tensor core 22%, DRAM 27%; a third of a block's clocks go into the drains (one
+// per eight tiles), half into conversion and reading, the rest into the barrier and the waits.
 __global__ void __launch_bounds__(CNT, 2) contract_kernel(const double* __restrict__ props, size_t V, int spatial,
                                                           int nbx, double* __restrict__ partial) {
   extern __shared__ __align__(128) char smem[];
-  __shared__ int tmax[4][12];  // largest biased exponents of the tile: per quarter of it and propagator
+  __shared__ int tmax[2][4][12];  // largest biased exponents of a tile (by parity): per quarter of it and propagator
   __shared__ int Es[12];
   __shared__ __align__(8) unsigned long long bar, full[2];
   __shared__ unsigned taddr;
@@ -197,40 +201,53 @@ __global__ void __launch_bounds__(CNT, 2) contract_kernel(const double* __restri
   int summed = 0;     // components in the sums
   unsigned phase = 0; // commits waited for
   bool pending = false, ok = true;
-  int n = 0;
-  for (int tl = blockIdx.x; tl <= ntile + nbx - 1; tl += nbx, ++n) {  // one more round drains
-    const bool last = tl >= ntile;
-    double x[8];
-    int e = 0;
-    bool bad = false;
-    if (!last) {
-      ok = c_wait(smem_addr(&full[n & 1]), (n >> 1) & 1) && ok;
-      const char* raw = smem + C_OPER + (n & 1) * C_RAW + j * C_ROWP + 8 * prt + 16 * kp;
+  double x[8];        // this thread's components of the tile in hand
+  int e = 0;          // their warp's largest exponent
+  bool bad = false;   // the tile has a real that the sums cannot take
+  // tile number n of this block, from its raw buffer
+  auto take = [&](int tl, int n) {
+    ok = c_wait(smem_addr(&full[n & 1]), (n >> 1) & 1) && ok;
+    const char* raw = smem + C_OPER + (n & 1) * C_RAW + j * C_ROWP + 8 * prt + 16 * kp;
+    if ((tl + 1) * CT <= ncomp) {  // uniform
+#pragma unroll
+      for (int m = 0; m < 8; ++m) x[m] = *reinterpret_cast<const double*>(raw + 256 * m);
+    } else {
 #pragma unroll
       for (int m = 0; m < 8; ++m)
         x[m] = tl * CT + kp + 16 * m < ncomp ? *reinterpret_cast<const double*>(raw + 256 * m) : 0.0;
-      unsigned u = 0, any = 0;
-#pragma unroll
-      for (int m = 0; m < 8; ++m) {
-        u = max(u, (unsigned)__double2hiint(x[m]) & 0x7fffffffu);
-        any |= (unsigned)__double2loint(x[m]);
-      }
-      e = (int)(u >> 20);
-      const bool zero = (u | any) == 0;
-      e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
-      e = max(e, __shfl_xor_sync(0xffffffffu, e, 8));
-      e = max(e, __shfl_xor_sync(0xffffffffu, e, 16));
-      if ((lane & 25) == 0) tmax[warp / 3][j] = e;
-      bad = e > FX_EMAX || (!zero && e < FX_EMIN);
     }
-    // one barrier decides the ordinary case: the exponents fit and the sums have room
+    unsigned u = 0;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) u = max(u, (unsigned)__double2hiint(x[m]) & 0x7fffffffu);
+    e = (int)(u >> 20);
+    bool zero = false;
+    if (u == 0) {
+      unsigned any = 0;
+#pragma unroll
+      for (int m = 0; m < 8; ++m) any |= (unsigned)__double2loint(x[m]);
+      zero = any == 0;
+    }
+    e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
+    e = max(e, __shfl_xor_sync(0xffffffffu, e, 8));
+    e = max(e, __shfl_xor_sync(0xffffffffu, e, 16));
+    if ((lane & 25) == 0) tmax[n & 1][warp / 3][j] = e;
+    bad = e > FX_EMAX || (!zero && e < FX_EMIN);
+  };
+  // one barrier per tile: the operand tile is written, and the next tile is in registers (its raw buffer
+  // is free) and known to fit the exponents or not
+  take(blockIdx.x, 0);
+  bool flag = __syncthreads_or(bad || e != 0) != 0;
+  if (warp == 11 && (int)blockIdx.x + 2 * nbx < ntile) fetch(blockIdx.x + 2 * nbx, 0);
+  int n = 0;
+  for (int tl = blockIdx.x;; tl += nbx, ++n) {  // one more round drains
+    const bool last = tl >= ntile;
     bool direct = false, drain = last || summed + CT > CK;
-    if (__syncthreads_or(bad || (e >= E && e != 0) || drain)) {
-      direct = __syncthreads_or(bad) != 0;  // the tile in FP64, outside the sums
+    if (flag || drain) {
+      direct = __syncthreads_or(!last && bad) != 0;  // the tile in FP64, outside the sums
       drain = last || !direct;
       if (!last) {
 #pragma unroll
-        for (int m = 0; m < 4; ++m) e = max(e, tmax[m][j]);
+        for (int m = 0; m < 4; ++m) e = max(e, tmax[n & 1][m][j]);
       }
     }
     if (drain) {
@@ -325,18 +342,21 @@ __global__ void __launch_bounds__(CNT, 2) contract_kernel(const double* __restri
           acc = part ? fma(p.x, q.y, fma(-p.y, q.x, acc)) : fma(p.x, q.x, fma(p.y, q.y, acc));
         }
       }
-      if (warp == 11 && tl + 2 * nbx < ntile) fetch(tl + 2 * nbx, n & 1);  // (the barriers above follow the reads)
-      continue;
+    } else {
+      // ---- the tile's digits, once the tensor core has read the last ones
+      if (pending) {
+        ok = c_wait(smem_addr(&bar), phase & 1) && ok;
+        phase ^= 1;
+      }
+      c_store_row(smem + kp * C_LBO, 2 * j + prt, x, E == 0 ? FX_BAD : E);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    // ---- the tile's digits, once the tensor core has read the last ones
-    if (pending) {
-      ok = c_wait(smem_addr(&bar), phase & 1) && ok;
-      phase ^= 1;
-      pending = false;
-    }
-    c_store_row(smem + kp * C_LBO, 2 * j + prt, x, E == 0 ? FX_BAD : E);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
+    e = 0;
+    bad = false;
+    if (tl + nbx < ntile) take(tl + nbx, n + 1);
+    flag = __syncthreads_or(bad || (e >= E && e != 0)) != 0;
+    if (warp == 11 && tl + 3 * nbx < ntile) fetch(tl + 3 * nbx, (n + 1) & 1);
+    if (direct) continue;
     if (tid == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const unsigned a = smem_addr(smem);
@@ -348,7 +368,6 @@ __global__ void __launch_bounds__(CNT, 2) contract_kernel(const double* __restri
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(&bar))
                    : "memory");
     }
-    if (warp == 11 && tl + 2 * nbx < ntile) fetch(tl + 2 * nbx, n & 1);
     pending = true;
     summed += CT;
   }
