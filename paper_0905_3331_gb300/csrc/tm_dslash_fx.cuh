@@ -68,27 +68,64 @@ __device__ __forceinline__ int fx_exponent(const uint4 w[N]) {
   return any != 0 ? FX_BAD : 0;
 }
 
+// The same of the 2 N numbers of a lane pair.
+template <int N>
+__device__ __forceinline__ int fx_pair_exponent(const uint4 w[N]) {
+  unsigned m = 0;
+#pragma unroll
+  for (int k = 0; k < N; ++k) m = max(m, max(w[k].y & 0x7fffffffu, w[k].w & 0x7fffffffu));
+  m = max(m, __shfl_xor_sync(__activemask(), m, 1));
+  const int e = (int)(m >> 20);
+  if (e >= FX_EMIN && e <= FX_EMAX) return e;
+  unsigned any = m;  // both lanes of the pair come here
+#pragma unroll
+  for (int k = 0; k < N; ++k) any |= w[k].x | w[k].z;
+  any |= __shfl_xor_sync(3u << (threadIdx.x & 30), any, 1);
+  return any != 0 ? FX_BAD : 0;
+}
+
 // The exponent to convert at: that of a zero site (0) shifts everything out.
 __device__ __forceinline__ int fx_shift_exponent(int e) { return e == 0 ? FX_BAD : e; }
 
-// Six complex numbers at blocks ja .. ja + 2 and jb .. jb + 2 of site i of an FX half field (XIN) or an
-// FP64 half field, as integers, and their exponent (FX: the site's).
-template <bool XIN>
-__device__ __forceinline__ int fx_load(const char* in, int h, int i, int ja, int jb, cpx<fx> v[6]) {
+// What the hopping sum reads: an FP64 half field, an FX half field, or a canonical FP64 field.
+constexpr int FXS_HALF = 0, FXS_FX = 1, FXS_CANON = 2;
+// Canonical input: (t + z + y + parity) & 1 of the output site, that is the parity of its x (its
+// neighbours' sum is the same across t, z and y, the other across x), gamma5 applied or not, and whether
+// the field is 16-byte aligned.
+struct FxCanon {
+  int b, g5;
+  bool al;
+};
+
+// Six complex numbers at blocks ja .. ja + 2 and jb .. jb + 2 of site i (canonical: its lexicographic
+// index), as integers, and the site's exponent.
+template <int SRC>
+__device__ __forceinline__ int fx_load(const char* in, int h, int i, int ja, int jb, cpx<fx> v[6], const FxCanon& canon) {
   uint4 w[6];
-  const uint4* p = reinterpret_cast<const uint4*>(in) + i;
+  if (SRC == FXS_CANON) {
+    const double* p = reinterpret_cast<const double*>(in) + (size_t)i * 24;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) w[k] = __ldg(p + (size_t)(ja + k) * h);
+    for (int k = 0; k < 6; ++k) {
+      const double2 d = canon_load(p + 2 * (k < 3 ? ja + k : jb + k - 3), canon.al);
+      const unsigned m = (k >= 3 && canon.g5) ? 0x80000000u : 0u;  // the partner is a lower spin
+      w[k] = make_uint4((unsigned)__double2loint(d.x), (unsigned)__double2hiint(d.x) ^ m, (unsigned)__double2loint(d.y),
+                        (unsigned)__double2hiint(d.y) ^ m);
+    }
+  } else {
+    const uint4* p = reinterpret_cast<const uint4*>(in) + i;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) w[3 + k] = __ldg(p + (size_t)(jb + k) * h);
+    for (int k = 0; k < 3; ++k) w[k] = __ldg(p + (size_t)(ja + k) * h);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) w[3 + k] = __ldg(p + (size_t)(jb + k) * h);
+  }
   int e;
-  if (XIN) {
+  if (SRC == FXS_FX) {
     e = __ldg(fx_exps(in, h) + i);
 #pragma unroll
     for (int k = 0; k < 6; ++k)
       v[k] = mk<fx>((fx)(((unsigned long long)w[k].y << 32) | w[k].x), (fx)(((unsigned long long)w[k].w << 32) | w[k].z));
   } else {
-    e = fx_exponent<6>(w);
+    e = fx_pair_exponent<6>(w);  // the site's: its twelve components are the lane pair's
     const int es = fx_shift_exponent(e);
 #pragma unroll
     for (int k = 0; k < 6; ++k) v[k] = mk<fx>(fx_from(w[k].x, w[k].y, es), fx_from(w[k].z, w[k].w, es));
@@ -262,22 +299,14 @@ __device__ __forceinline__ void fx_hop_apply(int mu, int q, int one, FxAcc& A, c
 }
 
 // One hop read into registers and applied.
-template <bool XIN, int S>
+template <int SRC, int S>
 __device__ __forceinline__ void fx_hop(int mu, int q, int one, FxAcc& A, const char* in, int h, int nbi, const char* slab,
-                                       int li, bool negate) {
+                                       int li, bool negate, const FxCanon& canon) {
   const RawWords<FX_LINK_BYTES> U = load_raw<FX_LINK_BYTES>(slab, h, li);
   const bool tz = mu == 0 || mu == 3;
   cpx<fx> v[6];
-  int e = fx_load<XIN>(in, h, nbi, 3 * q, tz ? 6 + 3 * q : 9 - 3 * q, v);
-  if (!XIN) {  // the site's exponent from the lane pair; both lanes keep the same E
-    const int eo = __shfl_xor_sync(__activemask(), e, 1);
-    if (eo > e) {
-      const int d = min(eo - e, 63);
-#pragma unroll
-      for (int k = 0; k < 6; ++k) v[k] = mk<fx>(v[k].re >> d, v[k].im >> d);
-      e = eo;
-    }
-  }
+  const int e = fx_load<SRC>(in, h, SRC == FXS_CANON ? 2 * nbi + (mu == 1 ? 1 - canon.b : canon.b) : nbi, 3 * q,
+                       tz ? 6 + 3 * q : 9 - 3 * q, v, canon);
   fx_hop_apply<S>(mu, q, one, A, v, e,
                   [&](int k) { return make_uint4(U.w[4 * k], U.w[4 * k + 1], U.w[4 * k + 2], U.w[4 * k + 3]); }, negate);
 }
@@ -306,9 +335,9 @@ __device__ __forceinline__ void fx_neighbours(const Geom& g, int cb, const SiteC
 // as one loop over the same code (what differs between them are signs and uniform branches): unrolled,
 // the sum was ~100 kB of instructions and the kernel waited for instruction fetch (16^3 x 32
 // 97-130 us, 4^4 38 us).
-template <bool XIN>
+template <int SRC>
 __device__ __forceinline__ void fx_hops(FxAcc& A, int q, const Geom& g, int cb, const SiteCoord& c, const char* in,
-                                        const char* lf, const char* lo, int d0, int d1) {
+                                        const char* lf, const char* lo, int d0, int d1, const FxCanon& canon = {0, 0, true}) {
   const size_t slab = (size_t)FX_LINK_BYTES * g.h;
   const int one = fx_one();
 #pragma unroll 1
@@ -316,8 +345,8 @@ __device__ __forceinline__ void fx_hops(FxAcc& A, int q, const Geom& g, int cb, 
     int nf, nb;
     bool wf, wb;
     fx_neighbours(g, cb, c, mu, nf, nb, wf, wb);
-    fx_hop<XIN, +1>(mu, q, one, A, in, g.h, nf, lf + mu * slab, cb, mu == 0 && wf);
-    fx_hop<XIN, -1>(mu, q, one, A, in, g.h, nb, lo + mu * slab, nb, mu == 0 && wb);
+    fx_hop<SRC, +1>(mu, q, one, A, in, g.h, nf, lf + mu * slab, cb, mu == 0 && wf, canon);
+    fx_hop<SRC, -1>(mu, q, one, A, in, g.h, nb, lo + mu * slab, nb, mu == 0 && wb, canon);
   }
 }
 

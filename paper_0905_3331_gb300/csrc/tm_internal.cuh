@@ -1289,8 +1289,12 @@ tm_status unpack_full_parity(tm_lattice lat, int prec, double* dst_full, const v
                              int g5, cudaStream_t s);
 tm_status convert_half(tm_lattice lat, int prec_out, void* dst, int prec_in, const void* src,
                        cudaStream_t s);
+// the threads per site of a form were chosen by tm_set_hop_threads or TM_HOP_TPS
+bool hop_tps_fixed(tm_lattice lat, int prec, int nreal);
+
 // out = M(f) in (eq. eo0), or gamma5 M(f) gamma5 in with g5, on canonical FP64 device fields (nrhs of them);
-// scratch holds the FX form of `per` fields at a time, full_fx_bytes(h) each (tm_operator_fx.cu)
+// scratch holds the FX form of `per` fields at a time, full_fx_bytes(h) each (tm_operator_fx.cu; small
+// fields are not brought to it)
 inline size_t full_fx_bytes(size_t h) { return (2 * fx_field_bytes(h) + 255) / 256 * 256; }
 tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g5, int nrhs, void* scratch, int per,
                      cudaStream_t s);

@@ -348,6 +348,10 @@ static int env_tps() {
   return (v == 1 || v == 2 || v == 4 || v == TM_HOP_PIPELINED || v == TM_HOP_PAIRED) ? v : 0;
 }
 
+bool hop_tps_fixed(tm_lattice lat, int prec, int nreal) {
+  return lat->hop_tps_forced[prec][link_index(nreal)] != 0 || env_tps() != 0;
+}
+
 // The choices made so far in this process.
 struct TuneChoice {
   int device, T, L, prec, nreal, tps;

@@ -9,10 +9,11 @@
 // call (most of it the hopping launch, latency bound as in tm_dslash_fx.cuh; 2.0 GB a call are 297 us of
 // HBM); 8^4 41 -> 16 us (two launches instead of six).
 //
-// One thread pair per site takes the next hop's neighbour and link into shared memory (cp.async) while it
+// The hopping launch takes the next hop's neighbour and link into shared memory (cp.async) while it
 // computes this one (fx_hops_staged): 32^3 x 64 1226 -> 1124 us, two fields of 20 x 14^3 79.9 -> 77.7.
-// Several pairs per site (small lattices) read into registers: they have more hops in flight as it is,
-// and staging cost 3 % there.
+//
+// Small lattices take one launch, which converts the canonical neighbours as it reads them: 8^4 16 -> 10
+// us (the rule and its figures are at CANON_SITES).
 #include "tm_hop_fx.cuh"
 
 namespace tmq {
@@ -45,16 +46,18 @@ __global__ void __launch_bounds__(128) full_to_fx_kernel(const Geom g, const dou
   const_cast<int*>(fx_exps(o, g.h))[cb] = e;
 }
 
-// out = D (c H in + E in) on both parities (blockIdx.y) of right-hand side blockIdx.z; D c real.
-template <int P>
+// out = D (c H in + E in) on both parities (blockIdx.y) of right-hand side blockIdx.z; D c real.  CANON: the
+// hopping sum reads the canonical field itself, with P thread pairs per site; otherwise its FX form fxin,
+// staged, with one.
+template <int P, bool CANON>
 __global__ void __launch_bounds__(fx_nt(P), HOP_FX_WARPS * 32 / fx_nt(P))
     full_fx_kernel(const Geom g, const char* __restrict__ links, const char* __restrict__ fxin, size_t fx_stride,
                    const double* __restrict__ in, double* __restrict__ out, const EpiCoef coef, int g5, bool al_in,
                    bool al_out) {
   constexpr int SPB = fx_spb(P), NT = fx_nt(P), WPP = NT / 32 / P;
-  constexpr bool STAGED = P == 1;
+  static_assert(CANON || P == 1);
   constexpr int TILE = SPB * CANON_TILE * 16, SUMS = P > 1 ? P * SPB * 2 * 19 * 8 : 0;
-  constexpr int STAGE = STAGED ? SPB * 2 * FX_STAGE * 16 : 0;
+  constexpr int STAGE = CANON ? 0 : SPB * 2 * FX_STAGE * 16;
   constexpr int SMEM = STAGE > TILE ? STAGE : (SUMS > TILE ? SUMS : TILE);
   // the staged hops or the parts' sums, then the results
   __shared__ __align__(16) char smem[SMEM];
@@ -79,10 +82,11 @@ __global__ void __launch_bounds__(fx_nt(P), HOP_FX_WARPS * 32 / fx_nt(P))
   A.bad = false;
   if (active) {
     const SiteCoord c = site_of(g, cb, parity);
-    if constexpr (STAGED)
-      fx_hops_staged<SPB>(A, q, g, cb, c, src, lf, lo, 0, 4, reinterpret_cast<uint4*>(smem), lane2 >> 1);
+    if constexpr (CANON)
+      fx_hops<FXS_CANON>(A, q, g, cb, c, reinterpret_cast<const char*>(inr), lf, lo, part * (4 / P), (part + 1) * (4 / P),
+                         FxCanon{(c.t + c.z + c.y + parity) & 1, g5, al_in});
     else
-      fx_hops<true>(A, q, g, cb, c, src, lf, lo, part * (4 / P), (part + 1) * (4 / P));
+      fx_hops_staged<SPB>(A, q, g, cb, c, src, lf, lo, 0, 4, reinterpret_cast<uint4*>(smem), lane2 >> 1);
   }
   if constexpr (P > 1) fx_merge<P, SPB>(A, part, lane2, reinterpret_cast<fx*>(smem));
   __syncthreads();
@@ -115,6 +119,19 @@ __global__ void __launch_bounds__(fx_nt(P), HOP_FX_WARPS * 32 / fx_nt(P))
   }
 }
 
+// Which form of the second launch, from the sites of both parities and all right-hand sides, by
+// measurement (one field unless said; us, FX form | canonical form with 1, 2, 4 pairs per site):
+//   4^4 13.7 | 14.8 10.3 10.3      8^4 15.6 | 16.4 12.3 10.3      8^3 x 16 17.3 | 16.4 14.3 12.3
+//   10^3 x 16 22.5 | 20.5 18.5 21.8            3 fields of 8^3 x 16 26.7 | 24.6 25.7 30.4
+//   12^3 x 24 37.8 | 36.9 36.6 44.4            14^3 x 20 45.1 | 42.6 44.4 55.4
+//   2 fields of 14^3 x 20 73.8 | 76.0 80.0 104.5      16^3 x 32 90.1 | 97.5 102.6 129.0
+// Small: the launch and the pass over the FX form cost more than converting each neighbour as it is read,
+// eight times over.  The pairs per site are as many as one field fits on the chip in a wave of 16 warps
+// per SM.  With one pair both forms give the same bits, so that a field's result does not depend on the
+// right-hand sides beside it; with more, the canonical form serves any number of them.
+constexpr size_t CANON_SITES = 65536;
+constexpr size_t WAVE_LANES = 152 * 16 * 32;
+
 tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g5, int nrhs, void* scratch, int per,
                      cudaStream_t s) {
   tm_status st = ensure_links(lat, TM_F64, 18, s);
@@ -134,19 +151,25 @@ tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g
     const int n = nrhs - r < per ? nrhs - r : per;
     const double* src = in + (size_t)r * lat->V * 24;
     double* dst = out + (size_t)r * lat->V * 24;
-    full_to_fx_kernel<<<dim3((unsigned)((lat->V + 127) / 128), n), 128, 0, s>>>(g, src, fxs, stride, g5, al_in);
-    count_launch();
-#define TM_FULL(P)                                                                                             \
-  full_fx_kernel<P><<<dim3((g.h + fx_spb(P) - 1) / fx_spb(P), 2, n), fx_nt(P), 0, s>>>(g, links, fxs, stride, src, dst, \
-                                                                                       c, g5, al_in, al_out)
-    const int tps = lat->hop_tps[TM_F64][link_index(18)];
-    if (tps == 2)
-      TM_FULL(2);
-    else if (tps == 4)
-      TM_FULL(4);
-    else
-      TM_FULL(1);
+#define TM_FULL_ARGS g, links, fxs, stride, src, dst, c, g5, al_in, al_out
+#define TM_FULL(P)                                                                                         \
+  full_fx_kernel<P, true><<<dim3((g.h + fx_spb(P) - 1) / fx_spb(P), 2, n), fx_nt(P), 0, s>>>(TM_FULL_ARGS)
+    int pairs = lat->hop_tps[TM_F64][link_index(18)];
+    if (!hop_tps_fixed(lat, TM_F64, 18)) pairs = lat->V * 8 <= WAVE_LANES ? 4 : (lat->V * 4 <= WAVE_LANES ? 2 : 1);
+    if (pairs > 1 || (size_t)n * lat->V <= CANON_SITES) {
+      if (pairs == 2)
+        TM_FULL(2);
+      else if (pairs == 4)
+        TM_FULL(4);
+      else
+        TM_FULL(1);
+    } else {
+      full_to_fx_kernel<<<dim3((unsigned)((lat->V + 127) / 128), n), 128, 0, s>>>(g, src, fxs, stride, g5, al_in);
+      count_launch();
+      full_fx_kernel<1, false><<<dim3((g.h + fx_spb(1) - 1) / fx_spb(1), 2, n), fx_nt(1), 0, s>>>(TM_FULL_ARGS);
+    }
 #undef TM_FULL
+#undef TM_FULL_ARGS
     count_launch();
     if ((st = cuda_check(cudaGetLastError(), "operator kernel launch")) != TM_OK) return st;
   }

@@ -91,3 +91,22 @@ def test_apply_D_of_many_right_hand_sides():
         for r in (0, 31, 32, 33):
             lat.apply_D(one, x[r])
             assert torch.equal(out[r], one)
+
+
+@pytest.mark.parametrize("T,L", [(2, 4), (10, 6), (16, 8), (16, 10), (24, 12)])
+def test_apply_D_of_a_field_beside_others(T, L):
+    """A field's result has the same bits alone and beside enough others to pass 65536 sites, for one,
+    two and four thread pairs per site; sites outside the fixed-point range and zero sites among them."""
+    n = 65536 // (T * L ** 3) + 1
+    with Lattice(T, L, 0.16, 0.01) as lat:
+        lat.set_gauge(torch.from_numpy(inputs.random_gauge(T, L, 0.5, 3)).cuda())
+        g = torch.Generator(device="cuda").manual_seed(5)
+        x = torch.randn((n, T, L, L, L, 4, 3), dtype=torch.complex128, device="cuda", generator=g)
+        scale = torch.tensor([0.0, 1e-306, 1e-20, 1.0, 1.0, 1.0, 1.0, 1e300], dtype=torch.float64, device="cuda")
+        x *= scale[torch.randint(8, (n, T, L, L, L, 1, 1), device="cuda", generator=g)]
+        out, one = torch.zeros_like(x), torch.zeros_like(x[0])
+        for dagger in (False, True):
+            lat.apply_D(out, x, dagger=dagger, nrhs=n)
+            for r in (0, n - 1):
+                lat.apply_D(one, x[r], dagger=dagger)
+                assert torch.equal(out[r], one)
