@@ -15,8 +15,9 @@ __device__ __forceinline__ void apply_g5(cpx<R> s[12]) {
 
 // Canonical records <-> a device half field, FNT sites per block through shared memory.  FULL: the sites
 // of parity p of a canonical full field (times gamma5 if g5), else a canonical half field [rhs][cb].
-// Bound by HBM: packing and unpacking two FP32 fields on 24^3 x 48 (382 MB) 163 -> 88 us; with a record
-// read or written by one thread, unpacking alone took 115 us.
+// Bound by HBM: packing and unpacking two FP32 fields on 24^3 x 48 (382 MB) 163 -> 73 us (36 each); with a
+// record read or written by one thread, unpacking alone took 115 us.  Packing copies asynchronously: through
+// registers its guarded loads followed one another (52 us, long scoreboard 24 cycles an issue).
 template <bool FULL>
 __device__ __forceinline__ void tile_index(const Geom& g, int first, int n, int p, unsigned* lex) {
   if (FULL && (int)threadIdx.x < n) lex[threadIdx.x] = (unsigned)lex_of_cb(g, first + threadIdx.x, p);
@@ -40,8 +41,9 @@ __global__ void __launch_bounds__(FNT) pack_kernel(const Geom g, const double* _
 #pragma unroll
   for (int j = 0; j < 12; ++j) {
     const int i = j * FNT + threadIdx.x;
-    if (i < n * 12) tile[i / 12 * CANON_TILE + i % 12] = canon_load(in + tile_offset<FULL>(first, i, lex), al);
+    if (i < n * 12) canon_to_shared(&tile[i / 12 * CANON_TILE + i % 12], in + tile_offset<FULL>(first, i, lex), al);
   }
+  canon_wait();
   __syncthreads();
   if ((int)threadIdx.x >= n) return;
   cpx<double> s[12];

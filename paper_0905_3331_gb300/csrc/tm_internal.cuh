@@ -204,6 +204,16 @@ __device__ __forceinline__ void canon_store(double* p, double2 v, bool al) {
     p[1] = v.y;
   }
 }
+// 16 bytes of a canonical record to shared memory: asynchronously where aligned (canon_wait makes this
+// thread's visible to it), so that all of a thread's copies are in flight and hold no registers.
+__device__ __forceinline__ void canon_to_shared(double2* dst, const double* src, bool al) {
+  if (al)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+  else
+    *dst = canon_load(src, false);
+}
+__device__ __forceinline__ void canon_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 inline bool canon_aligned(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
 
 // lexicographic index of site cb of parity p

@@ -10,7 +10,7 @@
 // HBM); 8^4 41 -> 16 us (two launches instead of six).
 //
 // The hopping launch takes the next hop's neighbour and link into shared memory (cp.async) while it
-// computes this one (fx_hops_staged): 32^3 x 64 1226 -> 1124 us, two fields of 20 x 14^3 79.9 -> 77.7.
+// computes this one (fx_hops_staged): 32^3 x 64 1226 -> 1112 us, two fields of 20 x 14^3 79.9 -> 77.5.
 //
 // Small lattices take one launch, which converts the canonical neighbours as it reads them: 8^4 16 -> 10
 // us (the rule and its figures are at CANON_SITES).
@@ -25,7 +25,8 @@ __global__ void __launch_bounds__(128) full_to_fx_kernel(const Geom g, const dou
   const size_t V = 2 * (size_t)g.h, first = (size_t)blockIdx.x * 128;
   const int n = (int)min((size_t)128, V - first);
   const double* src = in + ((size_t)blockIdx.y * V + first) * 24;
-  for (int i = threadIdx.x; i < n * 12; i += 128) tile[i / 12 * CANON_TILE + i % 12] = canon_load(src + 2 * (size_t)i, al);
+  for (int i = threadIdx.x; i < n * 12; i += 128) canon_to_shared(&tile[i / 12 * CANON_TILE + i % 12], src + 2 * (size_t)i, al);
+  canon_wait();
   __syncthreads();
   if ((int)threadIdx.x >= n) return;
   const size_t lex = first + threadIdx.x;
