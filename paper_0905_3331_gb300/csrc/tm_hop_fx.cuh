@@ -194,28 +194,45 @@ __device__ __forceinline__ void hop_sites_fx(const Geom g, const int out_parity,
     fx_finish(A, q, active, g, out_parity, cb, HalfInput{XIN ? static_cast<const char*>(fxa.in64) : inr}, lf, lo, acc,
               unit);
     // epilogue: o_s = D_s (c acc_s + E_s y_s) as (D_s c unit) acc_s + (D_s E_s) y_s; a real D c (every
-    // coefficient set but the inverse site term) takes half the products
+    // coefficient set but the inverse site term) takes half the products.  An FP64 instruction of a warp
+    // takes 80 clocks of its quarter of the SM, so the units and MODE 2's -alpha go into the coefficients
+    // and r is where the chains begin: K4 on 12^3 x 24 31.0 -> 28.6 us (20 of them without an epilogue).
+    const double m = MODE == 2 ? -(alpha_src ? alpha_sign * alpha_src[rhs].alpha : alpha_sign) : 1.0;
     const double cc = coef.c * unit;
-    const cpx<double> Du = mk(coef.d_up_re, coef.d_up_im), Dl = mk(coef.d_lo_re, coef.d_lo_im);
-    const cpx<double> DCu = mk(coef.d_up_re * cc, coef.d_up_im * cc), DCl = mk(coef.d_lo_re * cc, coef.d_lo_im * cc);
+    const cpx<double> Du = MODE == 2 ? mk(m * coef.d_up_re, m * coef.d_up_im) : mk(coef.d_up_re, coef.d_up_im);
+    const cpx<double> Dl = MODE == 2 ? mk(m * coef.d_lo_re, m * coef.d_lo_im) : mk(coef.d_lo_re, coef.d_lo_im);
     const bool real_d = coef.d_up_im == 0.0 && coef.d_lo_im == 0.0;
     const int kq[2] = {3 * q, 6 + 3 * q};  // this lane's blocks: kq[half] + k
+    char* outr = static_cast<char*>(out) + (size_t)rhs * out_stride;
     cpx<double> o[6];
+    if (MODE == 2) {
+#pragma unroll
+      for (int k = 0; k < 6; ++k) o[k] = mk(0.0, 0.0);
+      if (active) {
+        const double2* p = reinterpret_cast<const double2*>(outr) + cb;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+          const double2 t = p[(size_t)(kq[k / 3] + k % 3) * g.h];
+          o[k] = mk(t.x, t.y);
+        }
+      }
+    }
     if (HAS_Y) {
-      const cpx<double> Eu = mk(coef.e_up_re, coef.e_up_im), El = mk(coef.e_lo_re, coef.e_lo_im);
-      const cpx<double> DEu = Du * Eu, DEl = Dl * El;
-      cpx<double> yv[6];
+      cpx<double> Eu = mk(coef.e_up_re, coef.e_up_im), El = mk(coef.e_lo_re, coef.e_lo_im);
+      cpx<double> yv[6];  // in units of yu
 #pragma unroll
       for (int k = 0; k < 6; ++k) yv[k] = mk(0.0, 0.0);
       if (active) {
         const char* yr = static_cast<const char*>(y) + (size_t)rhs * y_stride;
         if (fxa.flags & FX_Y) {  // uniform
           const double yu = fx_stored_unit(__ldg(fx_exps(yr, g.h) + cb));
+          Eu = yu * Eu;
+          El = yu * El;
           const longlong2* p = reinterpret_cast<const longlong2*>(yr) + cb;
 #pragma unroll
           for (int k = 0; k < 6; ++k) {
             const longlong2 t = __ldg(p + (size_t)(kq[k / 3] + k % 3) * g.h);
-            yv[k] = mk((double)t.x * yu, (double)t.y * yu);
+            yv[k] = mk((double)t.x, (double)t.y);
           }
         } else {
           const double2* p = reinterpret_cast<const double2*>(yr) + cb;
@@ -226,56 +243,52 @@ __device__ __forceinline__ void hop_sites_fx(const Geom g, const int out_parity,
           }
         }
       }
+      if (MODE == 3) {
 #pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        if (MODE == 3) {
+        for (int k = 0; k < 6; ++k) {
           const cpx<double> t = cc * acc[k] + (k < 3 ? Eu : El) * yv[k];
           o[k] = (k < 3 ? Du : Dl) * t;
           const cpx<double> M = k < 3 ? mk(coef.m_up_re, coef.m_up_im) : mk(coef.m_lo_re, coef.m_lo_im);
           nrm += norm2(t - M * o[k]);
-        } else {
-          o[k] = (k < 3 ? DEu : DEl) * yv[k];
         }
-      }
-      if (MODE != 3) {
-        if (real_d) {
-#pragma unroll
-          for (int k = 0; k < 6; ++k) {
-            const double d = k < 3 ? DCu.re : DCl.re;
-            o[k] = mk(fma(d, acc[k].re, o[k].re), fma(d, acc[k].im, o[k].im));
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < 6; ++k) o[k] = o[k] + (k < 3 ? DCu : DCl) * acc[k];
-        }
-      }
-    } else if (real_d) {
-#pragma unroll
-      for (int k = 0; k < 6; ++k) o[k] = (k < 3 ? DCu.re : DCl.re) * acc[k];
-    } else {
-#pragma unroll
-      for (int k = 0; k < 6; ++k) o[k] = (k < 3 ? DCu : DCl) * acc[k];
-    }
-    char* outr = static_cast<char*>(out) + (size_t)rhs * out_stride;
-    if (MODE == 2) {
-      if (active) {
-        const double al = alpha_src ? alpha_sign * alpha_src[rhs].alpha : alpha_sign;
-        double2* p = reinterpret_cast<double2*>(outr) + cb;
-        cpx<double> r[6];
+      } else {
+        const cpx<double> DEu = real_d ? Du.re * Eu : Du * Eu, DEl = real_d ? Dl.re * El : Dl * El;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-          const double2 t = p[(size_t)(kq[k / 3] + k % 3) * g.h];
-          r[k] = mk(t.x, t.y) - al * o[k];
-          nrm += norm2(r[k]);
+          const cpx<double> DE = k < 3 ? DEu : DEl;
+          const double re = MODE == 2 ? fma(DE.re, yv[k].re, o[k].re) : DE.re * yv[k].re;
+          const double im = MODE == 2 ? fma(DE.re, yv[k].im, o[k].im) : DE.re * yv[k].im;
+          o[k] = mk(fma(-DE.im, yv[k].im, re), fma(DE.im, yv[k].re, im));
         }
+      }
+    }
+    if (MODE != 3) {
+      if (real_d) {
+        const double du = Du.re * cc, dl = Dl.re * cc;
 #pragma unroll
-        for (int k = 0; k < 6; ++k) p[(size_t)(kq[k / 3] + k % 3) * g.h] = make_double2(r[k].re, r[k].im);
+        for (int k = 0; k < 6; ++k) {
+          const double d = k < 3 ? du : dl;
+          o[k] = HAS_Y ? mk(fma(d, acc[k].re, o[k].re), fma(d, acc[k].im, o[k].im)) : mk(d * acc[k].re, d * acc[k].im);
+        }
+      } else {
+        const cpx<double> DCu = mk(Du.re * cc, Du.im * cc), DCl = mk(Dl.re * cc, Dl.im * cc);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) o[k] = HAS_Y ? o[k] + (k < 3 ? DCu : DCl) * acc[k] : (k < 3 ? DCu : DCl) * acc[k];
+      }
+    }
+    if (MODE == 1 || MODE == 2) {
+      if (active) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) nrm = fma(o[k].im, o[k].im, fma(o[k].re, o[k].re, nrm));
+      }
+    }
+    if (MODE == 2) {
+      if (active) {
+        double2* p = reinterpret_cast<double2*>(outr) + cb;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) p[(size_t)(kq[k / 3] + k % 3) * g.h] = make_double2(o[k].re, o[k].im);
       }
     } else {
-      if (MODE == 1 && active) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) nrm += norm2(o[k]);
-      }
       if (fxa.flags & FX_OUT) {  // uniform
         int e = active ? fx_exponent_f64<6>(o) : 0;
         e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
