@@ -191,7 +191,7 @@ __device__ __forceinline__ void hop_sites_fx(const Geom g, const int out_parity,
   if (part == 0) {
     cpx<double> acc[6];
     double unit;
-    fx_finish(A, q, active, g, out_parity, cb, HalfInput{XIN ? static_cast<const char*>(fxa.in64) : inr}, lf, lo, acc,
+    fx_finish(A, q, active, g, out_parity, cb, HalfInput{XIN ? nullptr : inr}, lf, lo, acc,
               unit);
     // epilogue: o_s = D_s (c acc_s + E_s y_s) as (D_s c unit) acc_s + (D_s E_s) y_s; a real D c (every
     // coefficient set but the inverse site term) takes half the products.  An FP64 instruction of a warp

@@ -1261,8 +1261,7 @@ bool is_device_pointer(const void* p);
 // tm_dslash_fx.cuh); the FX form of a half field takes fx_field_bytes(h) bytes.
 enum { FX_IN = 1, FX_OUT = 2, FX_Y = 4 };
 struct FxArgs {
-  int flags = 0;               // which of in, out, y are FX half fields
-  const void* in64 = nullptr;  // FX_IN: the FP64 field that in was made from, or null (inside a solver)
+  int flags = 0;  // which of in, out, y are FX half fields
 };
 __host__ __device__ inline size_t fx_field_bytes(size_t h) { return 196 * h; }
 
