@@ -67,6 +67,11 @@ static __device__ __noinline__ void hop_f64_general(const Geom& g, int out_parit
   }
 }
 
+// |x| == 1, on the words
+__device__ __forceinline__ bool fx_is_one(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7fffffffu) == 0x3ff00000u && __double2loint(x) == 0;
+}
+
 // acc = this lane's six components (spins q and 2 + q) of the sum A in FP64, with unit folded in by the
 // caller: real = acc unit.  All lanes of the warp call it (shuffles between the two lanes of a site).
 // in64: the FP64 input, if there is one.
@@ -253,11 +258,24 @@ __device__ __forceinline__ void hop_sites_fx(const Geom g, const int out_parity,
         }
       } else {
         const cpx<double> DEu = real_d ? Du.re * Eu : Du * Eu, DEl = real_d ? Dl.re * El : Dl * El;
+        // the Schur operator's D E = +-1 + i e_im on an FP64 y: the real part is a sign
+        const bool sign_re = MODE != 2 && fx_is_one(DEu.re) && fx_is_one(DEl.re);  // uniform
+        const int mu = __double2hiint(DEu.re) & 0x80000000, ml = __double2hiint(DEl.re) & 0x80000000;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
           const cpx<double> DE = k < 3 ? DEu : DEl;
-          const double re = MODE == 2 ? fma(DE.re, yv[k].re, o[k].re) : DE.re * yv[k].re;
-          const double im = MODE == 2 ? fma(DE.re, yv[k].im, o[k].im) : DE.re * yv[k].im;
+          double re, im;
+          if (MODE == 2) {
+            re = fma(DE.re, yv[k].re, o[k].re);
+            im = fma(DE.re, yv[k].im, o[k].im);
+          } else if (sign_re) {
+            const int m = k < 3 ? mu : ml;
+            re = __hiloint2double(__double2hiint(yv[k].re) ^ m, __double2loint(yv[k].re));
+            im = __hiloint2double(__double2hiint(yv[k].im) ^ m, __double2loint(yv[k].im));
+          } else {
+            re = DE.re * yv[k].re;
+            im = DE.re * yv[k].im;
+          }
           o[k] = mk(fma(-DE.im, yv[k].im, re), fma(DE.im, yv[k].re, im));
         }
       }

@@ -10,7 +10,8 @@
 // HBM); 8^4 41 -> 16 us (two launches instead of six).
 //
 // The hopping launch takes the next hop's neighbour and link into shared memory (cp.async) while it
-// computes this one (fx_hops_staged): 32^3 x 64 1226 -> 1112 us, two fields of 20 x 14^3 79.9 -> 77.5.
+// computes this one (fx_hops_staged): 32^3 x 64 1226 -> 1112 us, two fields of 20 x 14^3 79.9 -> 77.5;
+// with the real part of the site term as a sign, not a product, 1089 and 73.6.
 //
 // Small lattices take one launch, which converts the canonical neighbours as it reads them: 8^4 16 -> 10
 // us (the rule and its figures are at CANON_SITES).
@@ -47,7 +48,7 @@ __global__ void __launch_bounds__(128) full_to_fx_kernel(const Geom g, const dou
   const_cast<int*>(fx_exps(o, g.h))[cb] = e;
 }
 
-// out = D (c H in + E in) on both parities (blockIdx.y) of right-hand side blockIdx.z; D c real.  CANON: the
+// out = d H in + e in (d, e: coef's, d real) on both parities (blockIdx.y) of right-hand side blockIdx.z.  CANON: the
 // hopping sum reads the canonical field itself, with P thread pairs per site; otherwise its FX form fxin,
 // staged, with one.
 template <int P, bool CANON>
@@ -96,17 +97,20 @@ __global__ void __launch_bounds__(fx_nt(P), HOP_FX_WARPS * 32 / fx_nt(P))
     double unit;
     fx_finish(A, q, active, g, parity, cb, CanonInput{inr, 1 - parity, g5}, lf, lo, acc, unit);
     if (active) {
-      const cpx<double> DEu = mk(coef.d_up_re, 0.0) * mk(coef.e_up_re, coef.e_up_im);
-      const cpx<double> DEl = mk(coef.d_lo_re, 0.0) * mk(coef.e_lo_re, coef.e_lo_im);
-      const double cu = coef.d_up_re * coef.c * unit, cl = coef.d_lo_re * coef.c * unit;
+      // e = +-1 + i e_im: 6 FP64 instructions a component (80 clocks of the unit each) with the conversions
+      const double cu = coef.d_up_re * unit, cl = coef.d_lo_re * unit;
+      const int mu = __double2hiint(coef.e_up_re) & 0x80000000, ml = __double2hiint(coef.e_lo_re) & 0x80000000;
       const double* y = inr + lex_of_cb(g, cb, parity) * 24;
 #pragma unroll
       for (int k = 0; k < 6; ++k) {
         const int blk = (k < 3 ? 3 * q : 6 + 3 * q) + k % 3;
         const double2 t = canon_load(y + 2 * blk, al_in);
-        const cpx<double> e = (k < 3 ? DEu : DEl) * mk(t.x, t.y);
-        const double d = k < 3 ? cu : cl;
-        tile[site * CANON_TILE + blk] = make_double2(fma(d, acc[k].re, e.re), fma(d, acc[k].im, e.im));
+        const int m = k < 3 ? mu : ml;
+        const double im = k < 3 ? coef.e_up_im : coef.e_lo_im, d = k < 3 ? cu : cl;
+        const double sx = __hiloint2double(__double2hiint(t.x) ^ m, __double2loint(t.x));
+        const double sy = __hiloint2double(__double2hiint(t.y) ^ m, __double2loint(t.y));
+        tile[site * CANON_TILE + blk] =
+            make_double2(fma(d, acc[k].re, fma(-im, t.y, sx)), fma(d, acc[k].im, fma(im, t.x, sy)));
       }
     }
   }
@@ -126,6 +130,7 @@ __global__ void __launch_bounds__(fx_nt(P), HOP_FX_WARPS * 32 / fx_nt(P))
 //   10^3 x 16 22.5 | 20.5 18.5 21.8            3 fields of 8^3 x 16 26.7 | 24.6 25.7 30.4
 //   12^3 x 24 37.8 | 36.9 36.6 44.4            14^3 x 20 45.1 | 42.6 44.4 55.4
 //   2 fields of 14^3 x 20 73.8 | 76.0 80.0 104.5      16^3 x 32 90.1 | 97.5 102.6 129.0
+// (both a few per cent less since the site term's real part became a sign).
 // Small: the launch and the pass over the FX form cost more than converting each neighbour as it is read,
 // eight times over.  The pairs per site are as many as one field fits on the chip in a wave of 16 warps
 // per SM.  With one pair both forms give the same bits, so that a field's result does not depend on the
@@ -144,6 +149,12 @@ tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g
     c.e_lo_re = -c.e_lo_re;
     c.e_lo_im = -c.e_lo_im;
   }
+  c.e_up_re *= c.d_up_re;  // D (c H + E) multiplied out, D real
+  c.e_up_im *= c.d_up_re;
+  c.e_lo_re *= c.d_lo_re;
+  c.e_lo_im *= c.d_lo_re;
+  c.d_up_re *= c.c;
+  c.d_lo_re *= c.c;
   const char* links = static_cast<const char*>(lat->links[TM_F64][link_index(18)]);
   char* fxs = static_cast<char*>(scratch);
   const size_t stride = full_fx_bytes(lat->h);
