@@ -354,6 +354,89 @@ __device__ __forceinline__ void hop_pair(cpx<typename SpinorFmt<PREC>::real> acc
   }
 }
 
+// ---- FP16 storage: the pair of hops with the two projected spins as the lanes of packed FP32 operations.
+// Both spins take the same link: each link real, moved into both lanes, meets both in one instruction.  The
+// FP32 pipe's work is the same (a packed instruction holds it for two cycles), but the one-site FP16
+// kernels issued in 72% of all cycles and now issue a fifth less, with 16 warps per SM instead of 20-24:
+// FP16/8 on 48^3 x 96 374 -> 363 us, FP16/12 on 24^3 x 48 with 4 fields 90.1 -> 87.7.
+// Lower spins: lo holds (2, 3), lx (3, 2), as the directions deliver them.
+struct Acc16 {
+  cpx<f2> up[3], lo[3], lx[3];
+};
+
+template <int MU, int S>
+__device__ __forceinline__ void project16_lanes(const unsigned int w[13], bool negate, cpx<f2> h[3]) {
+  cpx<float> h0[3], h1[3];
+  project16<MU, S>(w, h0, h1);
+  const float n = __uint_as_float(w[12]);
+  const f2 f((MU == 0 && negate) ? -n : n);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) h[c] = mk<f2>(f * f2(h0[c].re, h1[c].re), f * f2(h0[c].im, h1[c].im));
+}
+
+// UP_FIRST, LOW_FIRST: the first pair that A.up, and A.lo (t, z) or A.lx (x, y), receives.
+template <int NREAL, int MU, bool UP_FIRST, bool LOW_FIRST>
+__device__ __forceinline__ void hop_pair16(Acc16& A, const void* in, int h, int nbf, const char* slabf, int lif, bool negf,
+                                           int nbb, const char* slabb, int lib, bool negb) {
+  constexpr int BYTES = NREAL * 2;
+  const RawWords<BYTES> rf = load_raw<BYTES>(slabf, h, lif);
+  const RawWords<BYTES> rb = load_raw<BYTES>(slabb, h, lib);
+  cpx<f2> u[3];
+  {
+    unsigned int w[13];
+    cpx<f2> v[3];
+    Mat3<float> U;
+    SpinorFmt<TM_F16>::load_words(in, h, nbf, w);
+    project16_lanes<MU, +1>(w, negf, v);
+    LinkRecon<float, __half, NREAL>::unpack(rf, U);
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const f2 nim = -v[b].im;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const f2 re(U.m[a][b].re), im(U.m[a][b].im);
+        u[a].re = fmadd(im, nim, b == 0 ? re * v[b].re : fmadd(re, v[b].re, u[a].re));
+        u[a].im = fmadd(im, v[b].re, b == 0 ? re * v[b].im : fmadd(re, v[b].im, u[a].im));
+      }
+    }
+  }
+  unsigned int w[13];
+  cpx<f2> v[3], s[3];
+  Mat3<float> U;
+  SpinorFmt<TM_F16>::load_words(in, h, nbb, w);
+  project16_lanes<MU, -1>(w, negb, v);
+  LinkRecon<float, __half, NREAL>::unpack(rb, U);
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    const f2 nre = -v[b].re;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {  // conj(U[b][a]) v[b]
+      const f2 re(U.m[b][a].re), im(U.m[b][a].im);
+      const cpx<f2> t = b == 0 ? u[a] : s[a];
+      s[a].re = fmadd(im, v[b].im, fmadd(re, v[b].re, t.re));
+      s[a].im = fmadd(im, nre, fmadd(re, v[b].im, t.im));
+    }
+  }
+  const f2 pm(1.f, -1.f), mp(-1.f, 1.f);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const cpx<f2> d = mk<f2>(fmadd(f2(-2.f), u[a].re, s[a].re), fmadd(f2(-2.f), u[a].im, s[a].im));  // u- - u+
+    A.up[a] = UP_FIRST ? s[a] : A.up[a] + s[a];
+    cpx<f2>& l = (MU == 0 || MU == 3) ? A.lo[a] : A.lx[a];
+    if (LOW_FIRST) {
+      if (MU == 0) l = d;
+      if (MU == 1) l = mk<f2>(d.im, -d.re);
+      if (MU == 2) l = mk<f2>(pm * d.re, pm * d.im);
+      if (MU == 3) l = mk<f2>(pm * d.im, mp * d.re);
+    } else {
+      if (MU == 0) l = l + d;
+      if (MU == 1) l = mk<f2>(l.re + d.im, fmadd(f2(-1.f), d.re, l.im));
+      if (MU == 2) l = mk<f2>(fmadd(pm, d.re, l.re), fmadd(pm, d.im, l.im));
+      if (MU == 3) l = mk<f2>(fmadd(pm, d.im, l.re), fmadd(mp, d.re, l.im));
+    }
+  }
+}
+
 // One hop.  Forward (S = +1): link U_mu(x) from the output parity's slab at the output site.
 // Backward (S = -1): link U_mu(x - mu^) from the other parity's slab at the neighbour's index,
 // applied as its adjoint -- the same stored link serves both hops, so the operator keeps
@@ -490,6 +573,7 @@ template <int PREC, int NREAL, int TPS>
 __device__ __forceinline__ void hop_part(cpx<typename SpinorFmt<PREC>::real> acc[12], const Geom& g, int cb,
                                          const SiteCoord& c, const int nb[8], const char* inr, const char* lf,
                                          const char* lo, size_t slab, int part) {
+  typedef typename SpinorFmt<PREC>::real R;
   const bool tfwd = (c.t == g.T - 1), tbwd = (c.t == 0);
   if constexpr (PREC == TM_DF64) {  // per hop (no fused multiply-add for double-float)
     if (TPS == 1 || part == 0 || (TPS == 2 && part == 0)) {
@@ -507,6 +591,30 @@ __device__ __forceinline__ void hop_part(cpx<typename SpinorFmt<PREC>::real> acc
     if (TPS == 1 || (TPS == 2 && part == 1) || (TPS == 4 && part == 3)) {
       hop_dir<PREC, NREAL, 3, +1>(acc, inr, g.h, nb[3], lf + 3 * slab, cb, false);
       hop_dir<PREC, NREAL, 3, -1>(acc, inr, g.h, nb[7], lo + 3 * slab, nb[7], false);
+    }
+  } else if constexpr (PREC == TM_F16) {
+    Acc16 A;
+    if (TPS == 4) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) A.lo[a] = A.lx[a] = mk<f2>(f2(0.f), f2(0.f));
+    }
+#define TM_PAIR16(MU, UF, LF, NF, NB)                                                                                   \
+  hop_pair16<NREAL, MU, UF, LF>(A, inr, g.h, nb[MU], lf + MU * slab, cb, NF, nb[4 + MU], lo + MU * slab, nb[4 + MU], NB);
+    if (TPS == 1 || part == 0) TM_PAIR16(0, true, true, tfwd, tbwd)
+    if (TPS == 1 || (TPS == 2 && part == 0)) TM_PAIR16(1, false, true, false, false)
+    if (TPS == 4 && part == 1) TM_PAIR16(1, true, true, false, false)
+    if (TPS == 1) TM_PAIR16(2, false, false, false, false)
+    if ((TPS == 2 && part == 1) || (TPS == 4 && part == 2)) TM_PAIR16(2, true, true, false, false)
+    if (TPS == 1) TM_PAIR16(3, false, false, false, false)
+    if (TPS == 2 && part == 1) TM_PAIR16(3, false, true, false, false)
+    if (TPS == 4 && part == 3) TM_PAIR16(3, true, true, false, false)
+#undef TM_PAIR16
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      acc[a] = mk<R>(A.up[a].re.v.x, A.up[a].im.v.x);
+      acc[3 + a] = mk<R>(A.up[a].re.v.y, A.up[a].im.v.y);
+      acc[6 + a] = mk<R>(A.lo[a].re.v.x + A.lx[a].re.v.y, A.lo[a].im.v.x + A.lx[a].im.v.y);
+      acc[9 + a] = mk<R>(A.lo[a].re.v.y + A.lx[a].re.v.x, A.lo[a].im.v.y + A.lx[a].im.v.x);
     }
   } else {
     // direction pairs; the first pair of a part writes the accumulator
@@ -532,7 +640,9 @@ __device__ __forceinline__ void hop_part(cpx<typename SpinorFmt<PREC>::real> acc
 // bound and the extra warps win over a few spilled bytes (FP32/12: 32^3 x 64 118 -> 113 us,
 // 16^3 x 32 18.9 -> 17.6 us per launch).  8- and 18-real links get 10 blocks (96 registers):
 // at 80 their direction pairs spilled 84-156 bytes (FP32/8 on 32^3 x 64: 115 -> 107 us with
-// 96, FP32/18: 157 -> 140 us).  FP64 and double-float keep their full budget (ALU bound).
+// 96, FP32/18: 157 -> 140 us).  FP16 storage, whose packed form holds each link real twice, gets 8 blocks
+// (128 registers; with 10 it spilled and gained nothing).  FP64 and double-float keep
+// their full budget (ALU bound).
 // The software-pipelined form holds two hops' words (72 more registers for FP32/12): a budget
 // for HOP_PIPE_BLOCKS blocks per SM.
 #ifndef HOP_PIPE_BLOCKS
@@ -541,12 +651,17 @@ __device__ __forceinline__ void hop_part(cpx<typename SpinorFmt<PREC>::real> acc
 #ifndef HOP_BLOCKS_12
 #define HOP_BLOCKS_12 12
 #endif
+#ifndef HOP_BLOCKS_F16
+#define HOP_BLOCKS_F16 8
+#endif
 #ifndef HOP_BLOCKS_OTHER
 #define HOP_BLOCKS_OTHER 10
 #endif
 constexpr int hop_min_blocks(int prec, int nreal, int tps, bool pipe) {
   return pipe ? HOP_PIPE_BLOCKS
-              : ((tps == 1 && (prec == TM_F32 || prec == TM_F16)) ? (nreal == 12 ? HOP_BLOCKS_12 : HOP_BLOCKS_OTHER) : 1);
+              : (tps != 1 ? 1
+                          : (prec == TM_F16 ? HOP_BLOCKS_F16
+                                            : (prec == TM_F32 ? (nreal == 12 ? HOP_BLOCKS_12 : HOP_BLOCKS_OTHER) : 1)));
 }
 
 // Which block of which right-hand side a block of the hopping kernel computes: the CUDA grid's
