@@ -16,6 +16,8 @@
 // are antiperiodic in time (Sec. 2.4): the hop across t = T-1 <-> 0 is multiplied by -1.
 #pragma once
 
+#include <type_traits>
+
 #include "tm_dslash_fx.cuh"
 #include "tm_internal.cuh"
 
@@ -569,7 +571,7 @@ __device__ __forceinline__ void hop_all_pipelined(cpx<typename SpinorFmt<PREC>::
 // are added in part order 0, 1, ..., and part q finishes the storage blocks
 // [NBLK q / TPS, NBLK (q + 1) / TPS) of the site.  More threads per site give more memory
 // requests in flight for lattices too small to fill the GPU with one thread per site.
-template <int PREC, int NREAL, int TPS>
+template <int PREC, int NREAL, int TPS, bool PACK>
 __device__ __forceinline__ void hop_part(cpx<typename SpinorFmt<PREC>::real> acc[12], const Geom& g, int cb,
                                          const SiteCoord& c, const int nb[8], const char* inr, const char* lf,
                                          const char* lo, size_t slab, int part) {
@@ -592,22 +594,15 @@ __device__ __forceinline__ void hop_part(cpx<typename SpinorFmt<PREC>::real> acc
       hop_dir<PREC, NREAL, 3, +1>(acc, inr, g.h, nb[3], lf + 3 * slab, cb, false);
       hop_dir<PREC, NREAL, 3, -1>(acc, inr, g.h, nb[7], lo + 3 * slab, nb[7], false);
     }
-  } else if constexpr (PREC == TM_F16) {
+  } else if constexpr (PACK) {
+    static_assert(PREC == TM_F16 && TPS == 1);
     Acc16 A;
-    if (TPS == 4) {
-#pragma unroll
-      for (int a = 0; a < 3; ++a) A.lo[a] = A.lx[a] = mk<f2>(f2(0.f), f2(0.f));
-    }
 #define TM_PAIR16(MU, UF, LF, NF, NB)                                                                                   \
   hop_pair16<NREAL, MU, UF, LF>(A, inr, g.h, nb[MU], lf + MU * slab, cb, NF, nb[4 + MU], lo + MU * slab, nb[4 + MU], NB);
-    if (TPS == 1 || part == 0) TM_PAIR16(0, true, true, tfwd, tbwd)
-    if (TPS == 1 || (TPS == 2 && part == 0)) TM_PAIR16(1, false, true, false, false)
-    if (TPS == 4 && part == 1) TM_PAIR16(1, true, true, false, false)
-    if (TPS == 1) TM_PAIR16(2, false, false, false, false)
-    if ((TPS == 2 && part == 1) || (TPS == 4 && part == 2)) TM_PAIR16(2, true, true, false, false)
-    if (TPS == 1) TM_PAIR16(3, false, false, false, false)
-    if (TPS == 2 && part == 1) TM_PAIR16(3, false, true, false, false)
-    if (TPS == 4 && part == 3) TM_PAIR16(3, true, true, false, false)
+    TM_PAIR16(0, true, true, tfwd, tbwd)
+    TM_PAIR16(1, false, true, false, false)
+    TM_PAIR16(2, false, false, false, false)
+    TM_PAIR16(3, false, false, false, false)
 #undef TM_PAIR16
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -640,7 +635,7 @@ __device__ __forceinline__ void hop_part(cpx<typename SpinorFmt<PREC>::real> acc
 // bound and the extra warps win over a few spilled bytes (FP32/12: 32^3 x 64 118 -> 113 us,
 // 16^3 x 32 18.9 -> 17.6 us per launch).  8- and 18-real links get 10 blocks (96 registers):
 // at 80 their direction pairs spilled 84-156 bytes (FP32/8 on 32^3 x 64: 115 -> 107 us with
-// 96, FP32/18: 157 -> 140 us).  FP16 storage, whose packed form holds each link real twice, gets 8 blocks
+// 96, FP32/18: 157 -> 140 us).  The packed FP16 form, which holds each link real twice, gets 8 blocks
 // (128 registers; with 10 it spilled and gained nothing).  FP64 and double-float keep
 // their full budget (ALU bound).
 // The software-pipelined form holds two hops' words (72 more registers for FP32/12): a budget
@@ -651,17 +646,20 @@ __device__ __forceinline__ void hop_part(cpx<typename SpinorFmt<PREC>::real> acc
 #ifndef HOP_BLOCKS_12
 #define HOP_BLOCKS_12 12
 #endif
-#ifndef HOP_BLOCKS_F16
-#define HOP_BLOCKS_F16 8
+#ifndef HOP_BLOCKS_PACKED
+#define HOP_BLOCKS_PACKED 8
 #endif
 #ifndef HOP_BLOCKS_OTHER
 #define HOP_BLOCKS_OTHER 10
 #endif
-constexpr int hop_min_blocks(int prec, int nreal, int tps, bool pipe) {
-  return pipe ? HOP_PIPE_BLOCKS
-              : (tps != 1 ? 1
-                          : (prec == TM_F16 ? HOP_BLOCKS_F16
-                                            : (prec == TM_F32 ? (nreal == 12 ? HOP_BLOCKS_12 : HOP_BLOCKS_OTHER) : 1)));
+// Packed FP16 arithmetic (hop_pair16): plain launches with one thread per site.  With an epilogue input or a
+// reduction the loads after the hops want the warps that its registers take: all launches packed, the
+// solves on 48^3 x 96 took 756 ms (8-real links) and 712 (12) against 732 and 700 with none.
+constexpr bool hop_packed(int prec, int tps, bool has_y, int mode) { return prec == TM_F16 && tps == 1 && !has_y && mode == 0; }
+constexpr int hop_min_blocks(int prec, int nreal, int tps, bool pipe, bool packed) {
+  return pipe     ? HOP_PIPE_BLOCKS
+         : packed ? HOP_BLOCKS_PACKED
+                  : ((tps == 1 && (prec == TM_F32 || prec == TM_F16)) ? (nreal == 12 ? HOP_BLOCKS_12 : HOP_BLOCKS_OTHER) : 1);
 }
 
 // Which block of which right-hand side a block of the hopping kernel computes: the CUDA grid's
@@ -693,6 +691,7 @@ __device__ __forceinline__ void hop_sites(const Geom g, const int out_parity, co
                                           const Blk B) {
   typedef typename SpinorFmt<PREC>::real R;
   typedef SpinorFmt<PREC> F;
+  constexpr bool PACK = std::is_same<Blk, GridBlock>::value && hop_packed(PREC, TPS, HAS_Y, MODE);
   constexpr int NT = SPB * TPS;            // threads per block (SPB sites per block)
   constexpr int WPP = (NT / 32) / TPS;     // warps per part
   constexpr int STRIDE = 25;               // 24 reals per site, padded against bank conflicts
@@ -719,7 +718,7 @@ __device__ __forceinline__ void hop_sites(const Geom g, const int out_parity, co
     if constexpr (PIPE)
       hop_all_pipelined<PREC, NREAL>(acc, g, cb, c, nb, inr, lf, lo, slab);
     else
-      hop_part<PREC, NREAL, TPS>(acc, g, cb, c, nb, inr, lf, lo, slab, part);
+      hop_part<PREC, NREAL, TPS, PACK>(acc, g, cb, c, nb, inr, lf, lo, slab, part);
   }
   // this thread's share of the site's storage blocks
   const int kb = (TPS == 1) ? 0 : F::CPB * ((F::NBLK * part) / TPS);
@@ -832,7 +831,7 @@ __device__ __forceinline__ void hop_sites(const Geom g, const int out_parity, co
 }
 
 template <int PREC, int NREAL, bool HAS_Y, int MODE, int TPS, bool PIPE>
-__global__ void __launch_bounds__(hop_spb(TPS) * TPS, hop_min_blocks(PREC, NREAL, TPS, PIPE)) hop_kernel(const Geom g, const int out_parity,
+__global__ void __launch_bounds__(hop_spb(TPS) * TPS, hop_min_blocks(PREC, NREAL, TPS, PIPE, hop_packed(PREC, TPS, HAS_Y, MODE))) hop_kernel(const Geom g, const int out_parity,
                                                      const char* __restrict__ links, const void* in,
                                                      size_t in_stride, void* out, size_t out_stride,
                                                      const void* y, size_t y_stride, const EpiCoef coef,
