@@ -133,15 +133,25 @@ __device__ __forceinline__ int fx_load(const char* in, int h, int i, int ja, int
   return e;
 }
 
-// Exponent of N FP64 complex numbers.
+// Exponent of N FP64 complex numbers, and of the 2 N of a lane pair.
 template <int N>
-__device__ __forceinline__ int fx_exponent_f64(const cpx<double> v[N]) {
-  uint4 w[N];
+__device__ __forceinline__ void fx_words(const cpx<double> v[N], uint4 w[N]) {
 #pragma unroll
   for (int k = 0; k < N; ++k)
     w[k] = make_uint4((unsigned)__double2loint(v[k].re), (unsigned)__double2hiint(v[k].re),
                       (unsigned)__double2loint(v[k].im), (unsigned)__double2hiint(v[k].im));
+}
+template <int N>
+__device__ __forceinline__ int fx_exponent_f64(const cpx<double> v[N]) {
+  uint4 w[N];
+  fx_words<N>(v, w);
   return fx_exponent<N>(w);
+}
+template <int N>
+__device__ __forceinline__ int fx_pair_exponent_f64(const cpx<double> v[N]) {
+  uint4 w[N];
+  fx_words<N>(v, w);
+  return fx_pair_exponent<N>(w);
 }
 __device__ __forceinline__ longlong2 fx_pack(cpx<double> v, int e) {
   e = fx_shift_exponent(e);

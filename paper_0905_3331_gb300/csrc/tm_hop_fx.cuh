@@ -308,8 +308,7 @@ __device__ __forceinline__ void hop_sites_fx(const Geom g, const int out_parity,
       }
     } else {
       if (fxa.flags & FX_OUT) {  // uniform
-        int e = active ? fx_exponent_f64<6>(o) : 0;
-        e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
+        const int e = fx_pair_exponent_f64<6>(o);  // the site's (a lane's six may be out of range by themselves)
         if (active) {
           longlong2* p = reinterpret_cast<longlong2*>(outr) + cb;
 #pragma unroll
