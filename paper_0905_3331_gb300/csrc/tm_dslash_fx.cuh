@@ -25,9 +25,12 @@
 // relative error of the sum 5.0e-17 on Gaussian fields (FP64 arithmetic: 1.3e-16), 3.9-5.6e-17 on point
 // sources, 5.5e-17 with time slices a factor e^1.5 apart, 6-8e-17 with sites of random size over e^40.
 //
-// A neighbour with a non-finite real, or whose largest real is outside [2^-894, 2^978) without being
-// zero throughout, has no FX form (exponent FX_BAD): its output site takes the FP64 form
-// (hop_f64_general) where the FP64 field is at hand, and is NaN where it is not (inside a solver).
+// A neighbour read from an FP64 field that has a non-finite real, or whose largest real is outside
+// [2^-894, 2^978) without being zero throughout, has no FX form (exponent FX_BAD): its output site takes
+// the FP64 form (hop_f64_general).  A site that a solver stores in FX form is held at the lowest exponent
+// if its largest real is below 2^-894 (to 2^-953; at least 2^370 below anything that a norm in FP64
+// sees), and is NaN to its readers if it has a non-finite real or one from 2^978 on, whose squares have
+// left FP64 as well.
 #pragma once
 
 #include "tm_internal.cuh"
@@ -68,8 +71,8 @@ __device__ __forceinline__ int fx_exponent(const uint4 w[N]) {
   return any != 0 ? FX_BAD : 0;
 }
 
-// The same of the 2 N numbers of a lane pair.
-template <int N>
+// The same of the 2 N numbers of a lane pair; TINY: the exponent where the largest is below 2^-894.
+template <int N, int TINY = FX_BAD>
 __device__ __forceinline__ int fx_pair_exponent(const uint4 w[N]) {
   unsigned m = 0;
 #pragma unroll
@@ -81,7 +84,7 @@ __device__ __forceinline__ int fx_pair_exponent(const uint4 w[N]) {
 #pragma unroll
   for (int k = 0; k < N; ++k) any |= w[k].x | w[k].z;
   any |= __shfl_xor_sync(3u << (threadIdx.x & 30), any, 1);
-  return any != 0 ? FX_BAD : 0;
+  return any == 0 ? 0 : (e > FX_EMAX ? FX_BAD : TINY);
 }
 
 // The exponent to convert at: that of a zero site (0) shifts everything out.
@@ -133,7 +136,7 @@ __device__ __forceinline__ int fx_load(const char* in, int h, int i, int ja, int
   return e;
 }
 
-// Exponent of N FP64 complex numbers, and of the 2 N of a lane pair.
+// Exponent of N FP64 complex numbers, and the one to store the 2 N of a lane pair with.
 template <int N>
 __device__ __forceinline__ void fx_words(const cpx<double> v[N], uint4 w[N]) {
 #pragma unroll
@@ -148,10 +151,10 @@ __device__ __forceinline__ int fx_exponent_f64(const cpx<double> v[N]) {
   return fx_exponent<N>(w);
 }
 template <int N>
-__device__ __forceinline__ int fx_pair_exponent_f64(const cpx<double> v[N]) {
+__device__ __forceinline__ int fx_stored_exponent(const cpx<double> v[N]) {
   uint4 w[N];
   fx_words<N>(v, w);
-  return fx_pair_exponent<N>(w);
+  return fx_pair_exponent<N, FX_EMIN>(w);
 }
 __device__ __forceinline__ longlong2 fx_pack(cpx<double> v, int e) {
   e = fx_shift_exponent(e);

@@ -308,7 +308,7 @@ __device__ __forceinline__ void hop_sites_fx(const Geom g, const int out_parity,
       }
     } else {
       if (fxa.flags & FX_OUT) {  // uniform
-        const int e = fx_pair_exponent_f64<6>(o);  // the site's (a lane's six may be out of range by themselves)
+        const int e = fx_stored_exponent<6>(o);  // the site's (a lane's six may be out of range by themselves)
         if (active) {
           longlong2* p = reinterpret_cast<longlong2*>(outr) + cb;
 #pragma unroll
