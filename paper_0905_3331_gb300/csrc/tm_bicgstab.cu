@@ -856,7 +856,7 @@ static tm_status solve_one_krylov(tm_lattice lat, double* x, const double* b, co
       // ||varphi_o - Mhat X|| up to the rounding of x_e (2 FP64 hopping launches instead of the
       // Schur residual's 2 followed by the reconstruction's 2)
       double rro = 0.0;
-      if ((st = reconstruct_xo(S, X, TM_F64, be, bo, bfull, x, T, w[6], w[7], &info->true_rel_residual, &rro)) != TM_OK)
+      if ((st = reconstruct_xo(S, X, be, bo, bfull, x, T, w[6], w[7], &info->true_rel_residual, &rro)) != TM_OK)
         return st;
       ++updates;
       if (bi_verbose())
@@ -898,7 +898,7 @@ static tm_status solve_one_krylov(tm_lattice lat, double* x, const double* b, co
   info->reliable_updates = updates;
   info->schur_rel_residual = std::sqrt(rr_true / bb);
   if (!reconstructed &&
-      (st = reconstruct_xo(S, X, TM_F64, be, bo, bfull, x, T, w[6], w[7], &info->true_rel_residual)) != TM_OK)
+      (st = reconstruct_xo(S, X, be, bo, bfull, x, T, w[6], w[7], &info->true_rel_residual)) != TM_OK)
     return st;
   info->status = converged ? TM_OK : TM_ERR_NOT_CONVERGED;
   if (!converged)

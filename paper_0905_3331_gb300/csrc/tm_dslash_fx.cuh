@@ -12,7 +12,7 @@
 // v = uh 2^32 + ul (LinkRecon<double, double, 18>).  A spinor site is 24 integers of a common exponent
 // e (a biased FP64 exponent: every real is below 2^(e - 1022)), real = V 2^(e - 1081), |V| < 2^59: the
 // site's largest real has six bits more than in FP64, and the others keep every bit down to the same
-// absolute place.  Half fields in this form are the storage format "FX" (TM_FX); FP64 fields are brought
+// absolute place.  Half fields in this form are called FX here; FP64 fields are brought
 // to it as they are read.  The sum has an exponent E of its own, at least e + 1 of every neighbour
 // added: a neighbour is shifted right by E - e, and the sum when E grows.  A projected real h so
 // shifted, |h| < 2^59, is hh 2^32 + hl, hl signed, and
@@ -40,6 +40,7 @@ namespace tmq {
 typedef long long fx;
 
 constexpr int FX_EMIN = 128, FX_EMAX = 2000;  // biased exponents of the fixed-point form
+constexpr int FX_BAD = 0x7fff;                // exponent of a site without a fixed-point form
 constexpr size_t FX_SITE_BYTES = 196;         // FX half field: longlong2 blocks [12][h], then int e[h]
 
 __device__ __forceinline__ const int* fx_exps(const char* base, int h) {
@@ -89,6 +90,11 @@ __device__ __forceinline__ int fx_pair_exponent(const uint4 w[N]) {
 
 // The exponent to convert at: that of a zero site (0) shifts everything out.
 __device__ __forceinline__ int fx_shift_exponent(int e) { return e == 0 ? FX_BAD : e; }
+
+// The unit 2^(e - 1081) of a site's integers.
+__device__ __forceinline__ double fx_stored_unit(int e) {
+  return e == FX_BAD ? __longlong_as_double(0x7ff8000000000000ll) : (e == 0 ? 0.0 : __hiloint2double((e - 58) << 20, 0));
+}
 
 // What the hopping sum reads: an FP64 half field, an FX half field, or a canonical FP64 field.
 constexpr int FXS_HALF = 0, FXS_FX = 1, FXS_CANON = 2;

@@ -135,12 +135,8 @@ tm_status unpack_full_parity(tm_lattice lat, int prec, double* dst_full, const v
                              cudaStream_t s) {
   const Geom& g = lat->geom;
   const unsigned nb = (unsigned)((g.h + FNT - 1) / FNT);
-  const char* in = static_cast<const char*>(src);
-  const bool al = canon_aligned(dst_full);
-  if (prec == TM_FX)
-    unpack_kernel<TM_FX, true><<<nb, FNT, 0, s>>>(g, in, 0, dst_full, parity, g5, al);
-  else
-    TM_PREC_SWITCH(prec, (unpack_kernel<P, true><<<nb, FNT, 0, s>>>(g, in, 0, dst_full, parity, g5, al)));
+  TM_PREC_SWITCH(prec, (unpack_kernel<P, true><<<nb, FNT, 0, s>>>(g, static_cast<const char*>(src), 0, dst_full, parity,
+                                                           g5, canon_aligned(dst_full))));
   count_launch();
   return cuda_check(cudaGetLastError(), "unpack kernel");
 }

@@ -550,28 +550,6 @@ struct SpinorFmt<TM_DF64> {
   __device__ static __forceinline__ float4 pack(const cpx<float>& z) { return make_float4(z.re, 0.f, z.im, 0.f); }
 };
 
-// FX form of an FP64 half field (tm_dslash_fx.cuh): longlong2 blocks [12][h], int e[h]; a real is
-// V 2^(e - 1081), NaN for e = FX_BAD.  Read-only here.
-constexpr int TM_FX = 4;
-constexpr int FX_BAD = 0x7fff;  // exponent of a site without a fixed-point form
-__device__ __forceinline__ double fx_stored_unit(int e) {
-  return e == FX_BAD ? __longlong_as_double(0x7ff8000000000000ll) : (e == 0 ? 0.0 : __hiloint2double((e - 58) << 20, 0));
-}
-template <>
-struct SpinorFmt<TM_FX> {
-  typedef double real;
-  template <typename R>
-  __device__ static __forceinline__ void load(const void* base, int h, int i, cpx<R> s[12]) {
-    const longlong2* p = static_cast<const longlong2*>(base);
-    const double unit = fx_stored_unit(__ldg(reinterpret_cast<const int*>(p + (size_t)12 * h) + i));
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      const longlong2 v = __ldg(p + (size_t)k * h + i);
-      s[k] = mk<R>((R)((double)v.x * unit), (R)((double)v.y * unit));
-    }
-  }
-};
-
 __host__ __device__ inline size_t spinor_bytes_per_site(int prec) {
   return prec == TM_F64 ? 192 : (prec == TM_F32 ? 96 : (prec == TM_F16 ? 52 : 192));
 }

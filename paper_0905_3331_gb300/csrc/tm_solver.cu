@@ -192,9 +192,10 @@ tm_status norm2_n(const Solver& S, int prec, int n, const void* x, double* out_h
 
 // A = Qhat^f Qhat^{-f} applied to `in` (precision prec, links nreal), result folded into
 // `r` as r -= alpha A in.  With `state` the iteration form is used (skip when done, alpha from
-// the state, FIN_CG_ALPHA / FIN_CG_RR); without it alpha = 1 and ||r||^2 goes to dscalars[0].
+// the state, FIN_CG_ALPHA / FIN_CG_RR); without it alpha = 1 and ||r||^2 goes to dscalars[0].  keep_w: W is
+// left as an FP64 field (Qhat^{-f} in), for a caller that returns it.
 tm_status normal_apply(const Solver& S, int prec, int nreal, const void* in, void* T, void* W, void* r,
-                       CGState* state) {
+                       CGState* state, bool keep_w) {
   tm_lattice lat = S.lat;
   const unsigned nb = hop_grid_blocks(lat->h, 4);  // enough for every threads-per-site choice
   tm_status st = ensure_reduce(lat, nb, 4);
@@ -205,7 +206,7 @@ tm_status normal_apply(const Solver& S, int prec, int nreal, const void* in, voi
   a.nrhs = 1;
   a.skip = state ? &state->done : nullptr;
   // FP64: T and W are FX half fields (tm_dslash_fx.cuh), the form that the FP64 hopping kernel computes in
-  const bool fx = prec == TM_F64 && nreal == 18;
+  const bool fx = prec == TM_F64 && nreal == 18, wfx = fx && !keep_w;
   // K1: T = (M_ee^{-f})^-1 H_eo in
   a.out_parity = 0;
   a.in = in;
@@ -214,7 +215,7 @@ tm_status normal_apply(const Solver& S, int prec, int nreal, const void* in, voi
   a.mode = 0;
   a.fx.flags = fx ? FX_OUT : 0;
   if ((st = hop_launch(lat, a, S.s)) != TM_OK) return st;
-  a.fx.flags = fx ? FX_IN | FX_OUT : 0;
+  a.fx.flags = (fx ? FX_IN : 0) | (wfx ? FX_OUT : 0);
   // K2: W = Qhat^{-f} in, <in, A in> = ||W||^2
   a.out_parity = 1;
   a.in = T;
@@ -235,6 +236,7 @@ tm_status normal_apply(const Solver& S, int prec, int nreal, const void* in, voi
   a.out = T;
   a.coef = epi_mdiag_inv_hop(S.mut, S.f);
   a.mode = 0;
+  a.fx.flags = (wfx ? FX_IN : 0) | (fx ? FX_OUT : 0);
   if ((st = hop_launch(lat, a, S.s)) != TM_OK) return st;
   // K4: r -= alpha Qhat^f W
   a.out_parity = 1;
@@ -243,7 +245,7 @@ tm_status normal_apply(const Solver& S, int prec, int nreal, const void* in, voi
   a.out = r;
   a.coef = epi_schur_q(lat->kappa, S.mut, S.f);
   a.mode = 2;
-  a.fx.flags = fx ? FX_IN | FX_Y : 0;
+  a.fx.flags = (fx ? FX_IN : 0) | (wfx ? FX_Y : 0);
   if (state) {
     a.alpha_src = state;
     a.alpha_sign = 1.0;
@@ -544,12 +546,13 @@ static tm_status run_stage(const Solver& S, const Stage& v, const CGState& init,
   return st;
 }
 
-// r = b' - A X in FP64 (r, X, b' FP64 odd fields; T, W FP64 temporaries); returns ||r||^2.
-tm_status true_residual(const Solver& S, void* r, const void* X, const void* bp, void* T, void* W,
-                               double* rr) {
+// r = b' - A X in FP64 (r, X, b' FP64 odd fields; T, W FP64 temporaries, W = Qhat^{-f} X in FP64 with
+// keep_w); returns ||r||^2.
+tm_status true_residual(const Solver& S, void* r, const void* X, const void* bp, void* T, void* W, double* rr,
+                        bool keep_w) {
   tm_status st = cuda_check(cudaMemcpyAsync(r, bp, S.hb[TM_F64], cudaMemcpyDeviceToDevice, S.s), "copy");
   if (st != TM_OK) return st;
-  if ((st = normal_apply(S, TM_F64, 18, X, T, W, r, nullptr)) != TM_OK) return st;
+  if ((st = normal_apply(S, TM_F64, 18, X, T, W, r, nullptr, keep_w)) != TM_OK) return st;
   if ((st = cuda_check(cudaMemcpyAsync(rr, S.lat->dscalars, sizeof(double), cudaMemcpyDeviceToHost, S.s),
                        "readback")) != TM_OK)
     return st;
@@ -669,17 +672,17 @@ tm_status reconstruct_check(const Solver& S, const void* X, const void* be, cons
   a.y = X;
   a.out = W;  // x_o
   a.coef = epi_schur_q(lat->kappa, S.mut, -S.f);
-  a.fx.flags = FX_IN | FX_OUT;
+  a.fx.flags = FX_IN;
   if ((st = hop_launch(lat, a, S.s)) != TM_OK) return st;
-  return reconstruct_xo(S, W, TM_FX, be, bo, bfull, x, T, R, Pv, true_rel, rr_odd);
+  return reconstruct_xo(S, W, be, bo, bfull, x, T, R, Pv, true_rel, rr_odd);
 }
 
-// x_e = (M_ee^f)^-1 (b_e + kappa H_eo x_o) from the odd solution xo (FP64, or FX form: xo_prec), written
-// with xo to the canonical field x; then ||b - M x|| / ||b|| in FP64 (T, R, Pv are FP64 scratch).  Two FP64
+// x_e = (M_ee^f)^-1 (b_e + kappa H_eo x_o) from the odd solution xo, written with xo to the
+// canonical field x; then ||b - M x|| / ||b|| in FP64 (T, R, Pv are FP64 scratch).  Two FP64
 // hopping launches: the first stores x_e and sums the even residual
 // ||b_e + kappa H_eo x_o - M_ee x_e||^2 from the same hopping sum; the second forms
 // (b - M x)_o = b_o - (M_oo x_o - kappa H_oe x_e) and its norm.  R is unused.
-tm_status reconstruct_xo(const Solver& S, const void* xo, int xo_prec, const void* be, const void* bo, double bfull, double* x,
+tm_status reconstruct_xo(const Solver& S, const void* xo, const void* be, const void* bo, double bfull, double* x,
                          void* T, void* R, void* Pv, double* true_rel, double* rr_odd) {
   (void)R;
   tm_lattice lat = S.lat;
@@ -697,8 +700,6 @@ tm_status reconstruct_xo(const Solver& S, const void* xo, int xo_prec, const voi
   a.out = T;  // x_e
   a.coef = epi_scaled_minv(S.mut, S.f, lat->kappa);
   a.mode = 3;
-  const bool xfx = xo_prec == TM_FX;
-  a.fx.flags = (xfx ? FX_IN : 0) | FX_OUT;
   a.red = Reduce{lat->partials, lat->counters, lat->dscalars, nullptr, FIN_STORE};
   if ((st = hop_launch(lat, a, s)) != TM_OK) return st;
   if ((st = cuda_check(cudaMemcpyAsync(Pv, bo, S.hb[TM_F64], cudaMemcpyDeviceToDevice, s), "copy")) != TM_OK)
@@ -709,7 +710,6 @@ tm_status reconstruct_xo(const Solver& S, const void* xo, int xo_prec, const voi
   a.y = W;
   a.out = Pv;
   a.mode = 2;  // Pv -= 1 * (M x)_o
-  a.fx.flags = FX_IN | (xfx ? FX_Y : 0);
   a.alpha_src = nullptr;
   a.alpha_sign = 1.0;
   a.red = Reduce{lat->partials, lat->counters, lat->dscalars + 1, nullptr, FIN_STORE};
@@ -722,8 +722,8 @@ tm_status reconstruct_xo(const Solver& S, const void* xo, int xo_prec, const voi
   const double rre = rr[0], rro = rr[1];
   *true_rel = bfull > 0.0 ? std::sqrt((rre + rro) / bfull) : 0.0;
   if (rr_odd) *rr_odd = rro;
-  if ((st = unpack_full_parity(lat, TM_FX, x, T, 0, 0, s)) != TM_OK) return st;
-  return unpack_full_parity(lat, xo_prec, x, W, 1, 0, s);
+  if ((st = unpack_full_parity(lat, TM_F64, x, T, 0, 0, s)) != TM_OK) return st;
+  return unpack_full_parity(lat, TM_F64, x, W, 1, 0, s);
 }
 
 tm_status launch_accumulate(const Solver& S, void* X, void* xs) {
@@ -749,8 +749,11 @@ tm_status cg_normal(const Solver& S, const tm_cg_params& P, const void* bp, doub
   double rr_true = bb;
   // starting residual R = b' - A X (X = 0 unless a guess is given)
   bool w_valid = false;  // W = Qhat^{-f} X of the current X (K2 of the last FP64 residual)
+  // FP64 mode: its last residual leaves x_o.  The mixed modes recompute it when they return it: an FP64 W
+  // costs their residuals ~30 % of K3 each.
+  const bool keep_w = P.mode == TM_CG_FP64;
   if (guess) {
-    if ((st = true_residual(S, R, X, bp, T, W, &rr_true)) != TM_OK) return st;
+    if ((st = true_residual(S, R, X, bp, T, W, &rr_true, keep_w)) != TM_OK) return st;
     w_valid = true;
   } else {
     if ((st = cuda_check(cudaMemsetAsync(X, 0, S.hb[TM_F64], s), "memset")) != TM_OK) return st;
@@ -775,7 +778,7 @@ tm_status cg_normal(const Solver& S, const tm_cg_params& P, const void* bp, doub
       if (fin.nonfinite) return set_error(TM_ERR_NONFINITE, "tm_solve_cg: non-finite value in the iteration");
       const bool progress = fin.iter > iters;
       iters = fin.iter;
-      if ((st = true_residual(S, R, X, bp, T, W, &rr_true)) != TM_OK) return st;
+      if ((st = true_residual(S, R, X, bp, T, W, &rr_true, keep_w)) != TM_OK) return st;
       w_valid = true;
       ++updates;
       trace_update(updates, rr_true, bb);
@@ -833,7 +836,7 @@ tm_status cg_normal(const Solver& S, const tm_cg_params& P, const void* bp, doub
         count_launch();
         w_valid = false;
       }
-      if ((st = true_residual(S, R, X, bp, T, W, &rr_true)) != TM_OK) return st;
+      if ((st = true_residual(S, R, X, bp, T, W, &rr_true, keep_w)) != TM_OK) return st;
       w_valid = true;
       ++updates;
       trace_update(updates, rr_true, bb);
@@ -932,7 +935,7 @@ tm_status cg_normal(const Solver& S, const tm_cg_params& P, const void* bp, doub
         rsrc = Rd;
         rprec = TM_DF64;
       } else {
-        if ((st = true_residual(S, R, X, bp, T, W, &rr_true)) != TM_OK) return st;
+        if ((st = true_residual(S, R, X, bp, T, W, &rr_true, keep_w)) != TM_OK) return st;
         w_valid = true;
       }
       ++updates;
@@ -943,7 +946,7 @@ tm_status cg_normal(const Solver& S, const tm_cg_params& P, const void* bp, doub
           break;
         }
         // confirm in FP64; if the double-float residual was too optimistic, carry on in FP64
-        if ((st = true_residual(S, R, X, bp, T, W, &rr_true)) != TM_OK) return st;
+        if ((st = true_residual(S, R, X, bp, T, W, &rr_true, keep_w)) != TM_OK) return st;
         w_valid = true;
         ++updates;
         trace_update(updates, rr_true, bb);
@@ -970,7 +973,7 @@ tm_status cg_normal(const Solver& S, const tm_cg_params& P, const void* bp, doub
   res->updates = updates;
   res->converged = converged;
   res->rr_true = rr_true;
-  res->xo_in_W = w_valid;
+  res->xo_in_W = w_valid && keep_w;
   res->pending = false;
   return TM_OK;
 }
@@ -1049,7 +1052,7 @@ static tm_status solve_one(tm_lattice lat, double* x, const double* b, const tm_
   if (reconstructed)
     st = TM_OK;
   else if (nr.xo_in_W)
-    st = reconstruct_xo(S, W, TM_FX, be, bo, bfull, x, T, R, Pv, &info->true_rel_residual);
+    st = reconstruct_xo(S, W, be, bo, bfull, x, T, R, Pv, &info->true_rel_residual);
   else
     st = reconstruct_check(S, X, be, bo, bfull, x, T, W, R, Pv, &info->true_rel_residual);
   if (st != TM_OK) return st;

@@ -23,16 +23,17 @@ unsigned blas_blocks(int h);
 tm_status norm2_half(const Solver& S, int prec, const void* x, double* out_host);
 // r -= alpha Qhat^f Qhat^{-f} in (iteration form with `state`, else alpha = 1 and ||r||^2 in dscalars[0])
 tm_status normal_apply(const Solver& S, int prec, int nreal, const void* in, void* T, void* W, void* r,
-                       CGState* state);
+                       CGState* state, bool keep_w = false);
 // r = b' - A X in FP64; ||r||^2 returned
-tm_status true_residual(const Solver& S, void* r, const void* X, const void* bp, void* T, void* W, double* rr);
+tm_status true_residual(const Solver& S, void* r, const void* X, const void* bp, void* T, void* W, double* rr,
+                        bool keep_w = false);
 CGState fresh_state(double rr, double stop2, int max_iter, int iter0, double delta2, double growth = 0.0);
 tm_status prepare_source(const Solver& S, const double* b, void* be, void* bo, void* bp, void* T, double* bb,
                          double* bfull);
 // rr_odd (optional): ||(b - M x)_o||^2, the odd part of the full residual
 tm_status reconstruct_check(const Solver& S, const void* X, const void* be, const void* bo, double bfull, double* x,
                             void* T, void* W, void* R, void* Pv, double* true_rel, double* rr_odd = nullptr);
-tm_status reconstruct_xo(const Solver& S, const void* xo, int xo_prec, const void* be, const void* bo, double bfull, double* x,
+tm_status reconstruct_xo(const Solver& S, const void* xo, const void* be, const void* bo, double bfull, double* x,
                          void* T, void* R, void* Pv, double* true_rel, double* rr_odd = nullptr);
 tm_status launch_accumulate(const Solver& S, void* X, void* xs);  // X (FP64) += xs (FP32); xs = 0
 
@@ -40,7 +41,7 @@ struct NormalResult {
   int iters, updates;
   bool converged;
   double rr_true;   // ||bp - A X||^2, recomputed in FP64 (the iterated one when `pending`)
-  bool xo_in_W;     // W holds Qhat^{-f} X for the final X in FX form (left by the last FP64 residual)
+  bool xo_in_W;     // W holds Qhat^{-f} X for the final X (left by the last FP64 residual)
   bool pending;     // the last sloppy stage reached the tolerance; X is not yet confirmed in FP64
 };
 // With defer_final (mixed modes, FP64 updates), a sloppy stage that reaches the tolerance ends
