@@ -72,13 +72,13 @@ __device__ __forceinline__ int fx_exponent(const uint4 w[N]) {
   return any != 0 ? FX_BAD : 0;
 }
 
-// The same of the 2 N numbers of a lane pair; TINY: the exponent where the largest is below 2^-894.
+// The same of the 2 N numbers of a lane pair, called by whole warps; TINY: the exponent where the largest is below 2^-894.
 template <int N, int TINY = FX_BAD>
 __device__ __forceinline__ int fx_pair_exponent(const uint4 w[N]) {
   unsigned m = 0;
 #pragma unroll
   for (int k = 0; k < N; ++k) m = max(m, max(w[k].y & 0x7fffffffu, w[k].w & 0x7fffffffu));
-  m = max(m, __shfl_xor_sync(__activemask(), m, 1));
+  m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
   const int e = (int)(m >> 20);
   if (e >= FX_EMIN && e <= FX_EMAX) return e;
   unsigned any = m;  // both lanes of the pair come here
@@ -350,7 +350,8 @@ __device__ __forceinline__ void fx_neighbours(const Geom& g, int cb, const SiteC
   }
 }
 
-// The hops of directions [d0, d1) of a site in lane q, A in units of 2^(E - 1079).  The directions run
+// The hops of directions [d0, d1) of a site in lane q, A in units of 2^(E - 1079).  Whole warps call it, lanes
+// past the last site with that site: its shuffles and warp barriers name every lane.  The directions run
 // as one loop over the same code (what differs between them are signs and uniform branches): unrolled,
 // the sum was ~100 kB of instructions and the kernel waited for instruction fetch (16^3 x 32
 // 97-130 us, 4^4 38 us).
@@ -417,7 +418,6 @@ __device__ __forceinline__ void fx_hops_staged(FxAcc& A, int q, const Geom& g, i
   const size_t slab = (size_t)FX_LINK_BYTES * g.h;
   const int one = fx_one();
   uint4* const s1 = stage + FX_STAGE * SITES;
-  const unsigned mask = __activemask();
   int nf, nb, e0, e1 = 0;
   bool wf, wb;
   fx_neighbours(g, cb, c, d0, nf, nb, wf, wb);
@@ -427,9 +427,9 @@ __device__ __forceinline__ void fx_hops_staged(FxAcc& A, int q, const Geom& g, i
     const int jb = (mu == 0 || mu == 3) ? 6 + 3 * q : 9 - 3 * q;
     fx_stage_hop<SITES>(s1, site, q, g.h, in, nb, lo + mu * slab, nb, jb, e1);
     asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncwarp(mask);
+    __syncwarp();
     fx_apply_staged<SITES, +1>(stage, site, mu, q, one, A, e0, mu == 0 && wf);
-    __syncwarp(mask);
+    __syncwarp();
     const bool wrap = mu == 0 && wb;
     if (mu + 1 < d1) {
       fx_neighbours(g, cb, c, mu + 1, nf, nb, wf, wb);
@@ -439,9 +439,9 @@ __device__ __forceinline__ void fx_hops_staged(FxAcc& A, int q, const Geom& g, i
     } else {
       asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
-    __syncwarp(mask);
+    __syncwarp();
     fx_apply_staged<SITES, -1>(s1, site, mu, q, one, A, e1, wrap);
-    __syncwarp(mask);
+    __syncwarp();
   }
 }
 

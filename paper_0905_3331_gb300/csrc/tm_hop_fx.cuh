@@ -114,7 +114,8 @@ __device__ __forceinline__ void fx_site(cpx<double> acc[6], int q, bool active, 
   for (int k = 0; k < 3; ++k) A.up[k] = A.s[k] = A.o[k] = mk<fx>(0, 0);
   A.E = 0;
   A.bad = false;
-  if (active) fx_hops<XIN>(A, q, g, cb, site_of(g, cb, out_parity), in, lf, lo, 0, 4);
+  const int site = min(cb, g.h - 1);
+  fx_hops<XIN>(A, q, g, site, site_of(g, site, out_parity), in, lf, lo, 0, 4);
   double unit;
   fx_finish(A, q, active, g, out_parity, cb, HalfInput{in64}, lf, lo, acc, unit);
 #pragma unroll
@@ -187,10 +188,8 @@ __device__ __forceinline__ void hop_sites_fx(const Geom g, const int out_parity,
   const size_t slab = (size_t)FX_LINK_BYTES * g.h;
   const char* lf = links + (size_t)(out_parity * 4) * slab;        // U_mu(x), x of this parity
   const char* lo = links + (size_t)((1 - out_parity) * 4) * slab;  // U_mu(y), y of the other parity
-  if (active) {
-    const SiteCoord c = site_of(g, cb, out_parity);
-    fx_hops<XIN>(A, q, g, cb, c, inr, lf, lo, part * (4 / P), (part + 1) * (4 / P));
-  }
+  const int site = min(cb, g.h - 1);
+  fx_hops<XIN>(A, q, g, site, site_of(g, site, out_parity), inr, lf, lo, part * (4 / P), (part + 1) * (4 / P));
   if constexpr (P > 1) fx_merge<P, SPB>(A, part, lane2, part_sum);
   double nrm = 0.0;
   if (part == 0) {

@@ -11,7 +11,8 @@
 //
 // The hopping launch takes the next hop's neighbour and link into shared memory (cp.async) while it
 // computes this one (fx_hops_staged): 32^3 x 64 1226 -> 1112 us, two fields of 20 x 14^3 79.9 -> 77.5;
-// with the real part of the site term as a sign, not a product, 1089 and 73.6.
+// with the real part of the site term as a sign, not a product, 1089 and 73.6; with whole warps in the loop
+// and constant masks 1067 and 71.7.
 //
 // Small lattices take one launch, which converts the canonical neighbours as it reads them: 8^4 16 -> 10
 // us (the rule and its figures are at CANON_SITES).
@@ -82,14 +83,13 @@ __global__ void __launch_bounds__(fx_nt(P), HOP_FX_WARPS * 32 / fx_nt(P))
   for (int k = 0; k < 3; ++k) A.up[k] = A.s[k] = A.o[k] = mk<fx>(0, 0);
   A.E = 0;
   A.bad = false;
-  if (active) {
-    const SiteCoord c = site_of(g, cb, parity);
-    if constexpr (CANON)
-      fx_hops<FXS_CANON>(A, q, g, cb, c, reinterpret_cast<const char*>(inr), lf, lo, part * (4 / P), (part + 1) * (4 / P),
-                         FxCanon{(c.t + c.z + c.y + parity) & 1, g5, al_in});
-    else
-      fx_hops_staged<SPB>(A, q, g, cb, c, src, lf, lo, 0, 4, reinterpret_cast<uint4*>(smem), lane2 >> 1);
-  }
+  const int cbs = min(cb, g.h - 1);
+  const SiteCoord c = site_of(g, cbs, parity);
+  if constexpr (CANON)
+    fx_hops<FXS_CANON>(A, q, g, cbs, c, reinterpret_cast<const char*>(inr), lf, lo, part * (4 / P), (part + 1) * (4 / P),
+                       FxCanon{(c.t + c.z + c.y + parity) & 1, g5, al_in});
+  else
+    fx_hops_staged<SPB>(A, q, g, cbs, c, src, lf, lo, 0, 4, reinterpret_cast<uint4*>(smem), site);
   if constexpr (P > 1) fx_merge<P, SPB>(A, part, lane2, reinterpret_cast<fx*>(smem));
   __syncthreads();
   if (part == 0) {
