@@ -636,7 +636,7 @@ extern "C" tm_status tm_apply_Dh(tm_lattice lat, double* out, const double* in, 
   const size_t hb2 = 2 * D.S.hb[TM_F64];
   void* w[4];
   for (int k = 0; k < 4; ++k) {
-    w[k] = workspace(lat, WS_APPLY_D + k, hb2, &st);
+    w[k] = workspace(lat, WS_APPLY_DH + k, hb2, &st);
     if (st != TM_OK) return st;
   }
   for (int r = 0; r < nrhs; ++r) {

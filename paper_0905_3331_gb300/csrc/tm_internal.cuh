@@ -1280,18 +1280,20 @@ tm_status convert_half(tm_lattice lat, int prec_out, void* dst, int prec_in, con
 bool hop_tps_fixed(tm_lattice lat, int prec, int nreal);
 
 // out = M(f) in (eq. eo0), or gamma5 M(f) gamma5 in with g5, on canonical FP64 device fields (nrhs of them);
-// scratch holds the FX form of `per` fields at a time, full_fx_bytes(h) each (tm_operator_fx.cu; small
-// fields are not brought to it)
+// scratch holds the FX form of `per` fields at a time, full_fx_bytes(h) each (tm_operator_fx.cu; few sites
+// are not brought to it)
 inline size_t full_fx_bytes(size_t h) { return (2 * fx_field_bytes(h) + 255) / 256 * 256; }
+// fields of the scratch that serves any nrhs, 0 if none needs one (once the FP64 links are built)
+int full_fx_fields(tm_lattice lat);
 tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g5, int nrhs, void* scratch, int per,
                      cudaStream_t s);
 tm_status diag_apply(tm_lattice lat, int prec, void* out, const void* in, int nrhs, double dur, double dui,
                      double dlr, double dli, cudaStream_t s);
-// Workspace slots: 0..17 CG solver, 22..25 tm_apply_D, 26 staged input, 27 staged output,
+// Workspace slots: 0..17 CG solver, 22..25 tm_apply_Dh, 26 staged input, 27 staged output,
 // 28 initial-guess work space, 29 contraction partials, 30 chronological-guess scalars,
-// 31 BiCGstab state; 18..20 BiCGstab vectors; 21 staged correlator matrices; 32 the FX form of an FP64
-// hopping launch's input.
-enum { WS_GAMMA = 21, WS_APPLY_D = 22, WS_STAGE_IN = 26, WS_STAGE_OUT = 27, WS_X0 = 28, WS_CHRONO = 30, WS_BISTATE = 31, WS_FX = 32 };
+// 31 BiCGstab state; 18..20 BiCGstab vectors; 21 staged correlator matrices; 32 the FX form of tm_apply_D's
+// input.
+enum { WS_GAMMA = 21, WS_APPLY_DH = 22, WS_STAGE_IN = 26, WS_STAGE_OUT = 27, WS_X0 = 28, WS_CHRONO = 30, WS_BISTATE = 31, WS_FULL_FX = 32 };
 // host-buffer staging through workspace slots
 const void* stage_in(tm_lattice lat, int slot, const void* src, size_t bytes, cudaStream_t s, tm_status* st);
 void* stage_out(tm_lattice lat, int slot, void* dst, size_t bytes, tm_status* st);

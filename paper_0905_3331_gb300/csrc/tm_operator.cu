@@ -1,7 +1,5 @@
 // tm_operator.cu -- the operator entry points: the hopping matrix H_{p,1-p} between half
 // fields (eq. eo2 blocks) and the full operator M of eq. eo0 on canonical fields.
-#include <algorithm>
-
 #include "tm_internal.cuh"
 
 namespace tmq {
@@ -55,10 +53,12 @@ tm_status tm_apply_D(tm_lattice lat, double* out, const double* in, int flavour,
   if (st != TM_OK) return st;
   double* dout = static_cast<double*>(stage_out(lat, WS_STAGE_OUT, out, fbytes * nrhs, &st));
   if (st != TM_OK) return st;
-  // the FX form of as many right-hand sides at a time as fit in 256 MiB, at least one
-  const size_t one = full_fx_bytes(lat->h);
-  const int per = (int)std::min<size_t>(nrhs, std::max<size_t>(1, ((size_t)256 << 20) / one));
-  void* w = workspace(lat, WS_APPLY_D, one * per, &st);
+  // the FX form of a fixed number of fields, whatever nrhs is: a buffer sized by nrhs would be freed and
+  // allocated anew by a call with more of them, under the feet of a captured one
+  if ((st = ensure_links(lat, TM_F64, 18, s)) != TM_OK) return st;
+  const int per = full_fx_fields(lat);
+  void* w = nullptr;
+  if (per > 0) w = workspace(lat, WS_FULL_FX, full_fx_bytes(lat->h) * per, &st);
   if (st != TM_OK) return st;
   // M^dag = g5 M(-f) g5
   if ((st = apply_full(lat, dout, din, dagger ? -flavour : flavour, dagger ? 1 : 0, nrhs, w, per, s)) != TM_OK) return st;

@@ -16,6 +16,8 @@
 //
 // Small lattices take one launch, which converts the canonical neighbours as it reads them: 8^4 16 -> 10
 // us (the rule and its figures are at CANON_SITES).
+#include <algorithm>
+
 #include "tm_hop_fx.cuh"
 
 namespace tmq {
@@ -137,6 +139,19 @@ __global__ void __launch_bounds__(fx_nt(P), HOP_FX_WARPS * 32 / fx_nt(P))
 // right-hand sides beside it; with more, the canonical form serves any number of them.
 constexpr size_t CANON_SITES = 65536;
 constexpr size_t WAVE_LANES = 152 * 16 * 32;
+// The FX form of as many fields at a time as fit in 256 MiB (1.4 million sites), at least one.  Smaller chunks
+// end in more last waves: 12 fields of 24 x 16^3 596 us with 1.4 million sites, 614 with 1.0, 629 with 0.5,
+// 686 with 0.25; of 20 x 14^3 336, 336, 350, 369.
+constexpr size_t FULL_FX_BYTES = (size_t)256 << 20;
+
+static int full_pairs(tm_lattice lat) {
+  if (hop_tps_fixed(lat, TM_F64, 18)) return lat->hop_tps[TM_F64][link_index(18)];
+  return lat->V * 8 <= WAVE_LANES ? 4 : (lat->V * 4 <= WAVE_LANES ? 2 : 1);
+}
+
+int full_fx_fields(tm_lattice lat) {
+  return full_pairs(lat) > 1 ? 0 : (int)std::max<size_t>(1, FULL_FX_BYTES / full_fx_bytes(lat->h));
+}
 
 tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g5, int nrhs, void* scratch, int per,
                      cudaStream_t s) {
@@ -159,16 +174,17 @@ tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g
   char* fxs = static_cast<char*>(scratch);
   const size_t stride = full_fx_bytes(lat->h);
   const bool al_in = canon_aligned(in), al_out = canon_aligned(out);
-  for (int r = 0; r < nrhs; r += per) {
-    const int n = nrhs - r < per ? nrhs - r : per;
+  const int pairs = full_pairs(lat);
+  for (int r = 0, n; r < nrhs; r += n) {
+    n = nrhs - r;
+    const bool canon = pairs > 1 || (size_t)n * lat->V <= CANON_SITES;
+    if (!canon) n = (n + (n + per - 1) / per - 1) / ((n + per - 1) / per);  // equal chunks of at most `per`
     const double* src = in + (size_t)r * lat->V * 24;
     double* dst = out + (size_t)r * lat->V * 24;
 #define TM_FULL_ARGS g, links, fxs, stride, src, dst, c, g5, al_in, al_out
 #define TM_FULL(P)                                                                                         \
   full_fx_kernel<P, true><<<dim3((g.h + fx_spb(P) - 1) / fx_spb(P), 2, n), fx_nt(P), 0, s>>>(TM_FULL_ARGS)
-    int pairs = lat->hop_tps[TM_F64][link_index(18)];
-    if (!hop_tps_fixed(lat, TM_F64, 18)) pairs = lat->V * 8 <= WAVE_LANES ? 4 : (lat->V * 4 <= WAVE_LANES ? 2 : 1);
-    if (pairs > 1 || (size_t)n * lat->V <= CANON_SITES) {
+    if (canon) {
       if (pairs == 2)
         TM_FULL(2);
       else if (pairs == 4)
