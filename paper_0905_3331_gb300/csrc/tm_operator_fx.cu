@@ -143,6 +143,7 @@ constexpr size_t WAVE_LANES = 152 * 16 * 32;
 // end in more last waves: 12 fields of 24 x 16^3 596 us with 1.4 million sites, 614 with 1.0, 629 with 0.5,
 // 686 with 0.25; of 20 x 14^3 336, 336, 350, 369.
 constexpr size_t FULL_FX_BYTES = (size_t)256 << 20;
+constexpr int MAX_FIELDS = 65535;  // of a launch: they are its gridDim.z (gridDim.y in the FX pass)
 
 static int full_pairs(tm_lattice lat) {
   if (hop_tps_fixed(lat, TM_F64, 18)) return lat->hop_tps[TM_F64][link_index(18)];
@@ -176,7 +177,7 @@ tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g
   const bool al_in = canon_aligned(in), al_out = canon_aligned(out);
   const int pairs = full_pairs(lat);
   for (int r = 0, n; r < nrhs; r += n) {
-    n = nrhs - r;
+    n = std::min(nrhs - r, MAX_FIELDS);
     const bool canon = pairs > 1 || (size_t)n * lat->V <= CANON_SITES;
     if (!canon) n = (n + (n + per - 1) / per - 1) / ((n + per - 1) / per);  // equal chunks of at most `per`
     const double* src = in + (size_t)r * lat->V * 24;

@@ -1,11 +1,12 @@
-"""The work buffer of the full operator: one size per lattice, whatever the number of right-hand sides."""
+"""The full operator with more right-hand sides than before: its work buffer has one size per lattice, and its
+launches stay within a grid's extents."""
 import pytest
 
 pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
 
-from paper_0905_3331_gb300 import Lattice, inputs  # noqa: E402
+from paper_0905_3331_gb300 import F64, LINK18, Lattice, inputs  # noqa: E402
 
 BIG = (20, 16)  # 81920 sites: the form with a work buffer
 
@@ -52,3 +53,18 @@ def test_captured_call_before_more_fields():
             many.replay()
         torch.cuda.synchronize()
         assert torch.equal(y[0], z[0]) and torch.equal(w, z)
+
+
+@pytest.mark.parametrize("threads", [0, 1])
+def test_more_fields_than_a_grid_dimension(threads):
+    """65600 fields on 2^4 against the same fields in three calls."""
+    n = 65600
+    with lattice(2, 2) as lat:
+        if threads:
+            lat.set_hop_threads(F64, LINK18, threads)
+        x = fields(n, 2, 2)
+        y, z = torch.zeros_like(x), torch.zeros_like(x)
+        lat.apply_D(y, x, nrhs=n)
+        for a, b in ((0, 30000), (30000, 60000), (60000, n)):
+            lat.apply_D(z[a:b], x[a:b], nrhs=b - a)
+        assert torch.equal(y, z)
