@@ -655,7 +655,11 @@ __device__ __forceinline__ void hop_part(cpx<typename SpinorFmt<PREC>::real> acc
 // Packed FP16 arithmetic (hop_pair16): plain launches with one thread per site.  With an epilogue input or a
 // reduction the loads after the hops want the warps that its registers take: all launches packed, the
 // solves on 48^3 x 96 took 756 ms (8-real links) and 712 (12) against 732 and 700 with none.
-constexpr bool hop_packed(int prec, int tps, bool has_y, int mode) { return prec == TM_F16 && tps == 1 && !has_y && mode == 0; }
+// Links of 18 reals have nothing to reconstruct: packed, 24^3 x 48 took 27.8 us against 27.3, three fields 73.3
+// against 72.4, and 4^4 with one thread per site 3.0 against 2.5 with two.
+constexpr bool hop_packed(int prec, int nreal, int tps, bool has_y, int mode) {
+  return prec == TM_F16 && nreal != 18 && tps == 1 && !has_y && mode == 0;
+}
 constexpr int hop_min_blocks(int prec, int nreal, int tps, bool pipe, bool packed) {
   return pipe     ? HOP_PIPE_BLOCKS
          : packed ? HOP_BLOCKS_PACKED
@@ -691,7 +695,7 @@ __device__ __forceinline__ void hop_sites(const Geom g, const int out_parity, co
                                           const Blk B) {
   typedef typename SpinorFmt<PREC>::real R;
   typedef SpinorFmt<PREC> F;
-  constexpr bool PACK = std::is_same<Blk, GridBlock>::value && hop_packed(PREC, TPS, HAS_Y, MODE);
+  constexpr bool PACK = std::is_same<Blk, GridBlock>::value && hop_packed(PREC, NREAL, TPS, HAS_Y, MODE);
   constexpr int NT = SPB * TPS;            // threads per block (SPB sites per block)
   constexpr int WPP = (NT / 32) / TPS;     // warps per part
   constexpr int STRIDE = 25;               // 24 reals per site, padded against bank conflicts
@@ -831,7 +835,7 @@ __device__ __forceinline__ void hop_sites(const Geom g, const int out_parity, co
 }
 
 template <int PREC, int NREAL, bool HAS_Y, int MODE, int TPS, bool PIPE>
-__global__ void __launch_bounds__(hop_spb(TPS) * TPS, hop_min_blocks(PREC, NREAL, TPS, PIPE, hop_packed(PREC, TPS, HAS_Y, MODE))) hop_kernel(const Geom g, const int out_parity,
+__global__ void __launch_bounds__(hop_spb(TPS) * TPS, hop_min_blocks(PREC, NREAL, TPS, PIPE, hop_packed(PREC, NREAL, TPS, HAS_Y, MODE))) hop_kernel(const Geom g, const int out_parity,
                                                      const char* __restrict__ links, const void* in,
                                                      size_t in_stride, void* out, size_t out_stride,
                                                      const void* y, size_t y_stride, const EpiCoef coef,
