@@ -18,6 +18,10 @@ __device__ __forceinline__ void apply_g5(cpx<R> s[12]) {
 // Bound by HBM: packing and unpacking two FP32 fields on 24^3 x 48 (382 MB) 163 -> 73 us (36 each); with a
 // record read or written by one thread, unpacking alone took 115 us.  Packing copies asynchronously: through
 // registers its guarded loads followed one another (52 us, long scoreboard 24 cycles an issue).
+// Double-float is bound by the FP64 units (24 splits or sums a site) and gains nothing from the tile where
+// the L2 takes what a record's accesses leave open: there a thread takes a whole record (!TILED).  Two
+// fields, tile and whole records: packing 16^3 x 32 28.9 and 27.0 us, 24^3 x 48 124 and 121; unpacking 12^3 x
+// 24 12.5 and 10.6, 16^3 x 32 22.7 and 20.8, but 24^3 x 48 92 and 122.
 template <bool FULL>
 __device__ __forceinline__ void tile_index(const Geom& g, int first, int n, int p, unsigned* lex) {
   if (FULL && (int)threadIdx.x < n) lex[threadIdx.x] = (unsigned)lex_of_cb(g, first + threadIdx.x, p);
@@ -27,13 +31,26 @@ __device__ __forceinline__ size_t tile_offset(int first, int i, const unsigned* 
   return 24 * (FULL ? (size_t)lex[i / 12] : (size_t)(first + i / 12)) + 2 * (i % 12);
 }
 
-template <int PREC, bool FULL>
+template <int PREC, bool FULL, bool TILED>
 __global__ void __launch_bounds__(FNT) pack_kernel(const Geom g, const double* __restrict__ src, char* __restrict__ dst,
                                                    size_t dstride, int p, int g5, bool al) {
-  __shared__ double2 tile[FNT * CANON_TILE];
-  __shared__ unsigned lex[FULL ? FNT : 1];
+  __shared__ double2 tile[TILED ? FNT * CANON_TILE : 1];
+  __shared__ unsigned lex[FULL && TILED ? FNT : 1];
   const int first = blockIdx.x * FNT, n = min(FNT, g.h - first), cb = first + threadIdx.x;
   const double* in = src + (size_t)blockIdx.y * g.h * 24;
+  cpx<double> s[12];
+  if constexpr (!TILED) {
+    if ((int)threadIdx.x >= n) return;
+    const double* rec = in + 24 * (FULL ? lex_of_cb(g, cb, p) : (size_t)cb);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const double2 v = canon_load(rec + 2 * k, al);
+      s[k] = mk(v.x, v.y);
+    }
+    if (FULL && g5) apply_g5(s);
+    SpinorFmt<PREC>::store(dst + blockIdx.y * dstride, g.h, cb, s);
+    return;
+  }
   if (FULL) {
     tile_index<FULL>(g, first, n, p, lex);
     __syncthreads();
@@ -46,25 +63,33 @@ __global__ void __launch_bounds__(FNT) pack_kernel(const Geom g, const double* _
   canon_wait();
   __syncthreads();
   if ((int)threadIdx.x >= n) return;
-  cpx<double> s[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) s[k] = mk(tile[threadIdx.x * CANON_TILE + k].x, tile[threadIdx.x * CANON_TILE + k].y);
   if (FULL && g5) apply_g5(s);
   SpinorFmt<PREC>::store(dst + blockIdx.y * dstride, g.h, cb, s);
 }
 
-template <int PREC, bool FULL>
+template <int PREC, bool FULL, bool TILED>
 __global__ void __launch_bounds__(FNT) unpack_kernel(const Geom g, const char* __restrict__ src, size_t sstride,
                                                      double* __restrict__ dst, int p, int g5, bool al) {
-  __shared__ double2 tile[FNT * CANON_TILE];
-  __shared__ unsigned lex[FULL ? FNT : 1];
+  __shared__ double2 tile[TILED ? FNT * CANON_TILE : 1];
+  __shared__ unsigned lex[FULL && TILED ? FNT : 1];
   const int first = blockIdx.x * FNT, n = min(FNT, g.h - first), cb = first + threadIdx.x;
   double* out = dst + (size_t)blockIdx.y * g.h * 24;
-  if (FULL) tile_index<FULL>(g, first, n, p, lex);
+  if (FULL && TILED) tile_index<FULL>(g, first, n, p, lex);
   if ((int)threadIdx.x < n) {
     cpx<double> s[12];
     SpinorFmt<PREC>::load(src + blockIdx.y * sstride, g.h, cb, s);
     if (FULL && g5) apply_g5(s);
+    if constexpr (!TILED) {  // (16-byte stores were no faster than the tile)
+      double* rec = out + 24 * (FULL ? lex_of_cb(g, cb, p) : (size_t)cb);
+#pragma unroll
+      for (int k = 0; k < 12; ++k) {
+        rec[2 * k] = s[k].re;
+        rec[2 * k + 1] = s[k].im;
+      }
+      return;
+    }
 #pragma unroll
     for (int k = 0; k < 12; ++k) tile[threadIdx.x * CANON_TILE + k] = make_double2(s[k].re, s[k].im);
   }
@@ -125,7 +150,7 @@ tm_status pack_full_parity(tm_lattice lat, int prec, void* dst, const double* sr
                            cudaStream_t s) {
   const Geom& g = lat->geom;
   const unsigned nb = (unsigned)((g.h + FNT - 1) / FNT);
-  TM_PREC_SWITCH(prec, (pack_kernel<P, true><<<nb, FNT, 0, s>>>(g, src_full, static_cast<char*>(dst), 0, parity, g5,
+  TM_PREC_SWITCH(prec, (pack_kernel<P, true, P != TM_DF64><<<nb, FNT, 0, s>>>(g, src_full, static_cast<char*>(dst), 0, parity, g5,
                                                          canon_aligned(src_full))));
   count_launch();
   return cuda_check(cudaGetLastError(), "pack kernel");
@@ -135,7 +160,7 @@ tm_status unpack_full_parity(tm_lattice lat, int prec, double* dst_full, const v
                              cudaStream_t s) {
   const Geom& g = lat->geom;
   const unsigned nb = (unsigned)((g.h + FNT - 1) / FNT);
-  TM_PREC_SWITCH(prec, (unpack_kernel<P, true><<<nb, FNT, 0, s>>>(g, static_cast<const char*>(src), 0, dst_full, parity,
+  TM_PREC_SWITCH(prec, (unpack_kernel<P, true, true><<<nb, FNT, 0, s>>>(g, static_cast<const char*>(src), 0, dst_full, parity,
                                                            g5, canon_aligned(dst_full))));
   count_launch();
   return cuda_check(cudaGetLastError(), "unpack kernel");
@@ -214,7 +239,7 @@ tm_status tm_pack_half(tm_lattice lat, tm_prec prec, void* dst, const double* sr
   const int h = lat->geom.h;
   dim3 grid((h + FNT - 1) / FNT, nrhs);
   const size_t stride = spinor_bytes_per_site(prec) * lat->h;
-  TM_PREC_SWITCH(prec, (pack_kernel<P, false><<<grid, FNT, 0, s>>>(lat->geom, static_cast<const double*>(d),
+  TM_PREC_SWITCH(prec, (pack_kernel<P, false, P != TM_DF64><<<grid, FNT, 0, s>>>(lat->geom, static_cast<const double*>(d),
                                                                    static_cast<char*>(dst), stride, 0, 0,
                                                                    canon_aligned(d))));
   count_launch();
@@ -232,9 +257,14 @@ tm_status tm_unpack_half(tm_lattice lat, tm_prec prec, double* dst, const void* 
   const int h = lat->geom.h;
   dim3 grid((h + FNT - 1) / FNT, nrhs);
   const size_t stride = spinor_bytes_per_site(prec) * lat->h;
-  TM_PREC_SWITCH(prec, (unpack_kernel<P, false><<<grid, FNT, 0, s>>>(lat->geom, static_cast<const char*>(src), stride,
-                                                                     static_cast<double*>(d), 0, 0,
-                                                                     canon_aligned(d))));
+  const char* in = static_cast<const char*>(src);
+  const bool al = canon_aligned(d);
+  // double-float fields that the L2 holds beside their canonical form (129 MB): whole records
+  if (prec == TM_DF64 && 2 * stride * nrhs <= ((size_t)126 << 20))
+    unpack_kernel<TM_DF64, false, false><<<grid, FNT, 0, s>>>(lat->geom, in, stride, static_cast<double*>(d), 0, 0, al);
+  else
+    TM_PREC_SWITCH(prec, (unpack_kernel<P, false, true><<<grid, FNT, 0, s>>>(lat->geom, in, stride,
+                                                                       static_cast<double*>(d), 0, 0, al)));
   count_launch();
   st = cuda_check(cudaGetLastError(), "tm_unpack_half");
   if (st != TM_OK) return st;
