@@ -90,13 +90,16 @@ __global__ void plans_init_kernel(Plans L) {
 // storage; serv = 1: the FP64 service of stopped systems, where K4's residual update uses alpha = 1
 // (r = b' - A X from r = b') and the reduction stores ||r||^2 in B.result.  A system that stopped
 // since the list was built (a breakdown in K2) is skipped.
-// FP32 / FP16 storage with one thread per site: 20 warps per SM (96 registers).  The launches wait for
-// loads (12 systems on 16^3 x 32, FP32/12: long scoreboard 6.2 of 10.3 cycles an issue at 20 warps, issue
-// slots 47 % busy, DRAM 35 %); with 16 warps of 128 registers the twelve solves took 66.7 ms, with 20
-// 63.5, with 24 (80 registers, spilled) 63.4.
+// FP32 / FP16 storage with one thread per site and 12- or 8-real links: 20 warps per SM (96 registers).  The
+// launches wait for loads (12 systems on 16^3 x 32, FP32/12: long scoreboard 6.2 of 10.3 cycles an issue at
+// 20 warps, issue slots 47 % busy, DRAM 35 %).  16 warps of 128 registers against 20 (24 with 80 registers
+// spilled), ms: those twelve solves FP32/12 49.5, 47.5; FP32/8 49.9, 48.3; FP16/12 57.3, 56.2; FP16/8 58.6,
+// 58.1; twelve on 12^3 x 24 FP32/12 19.0, 18.3.  18-real links keep 16 warps: FP32/18 50.2, 51.5, three
+// systems on 8^3 x 16 4.7, 5.0; FP16/18 58.5, 58.1 and 5.7, 5.9.
 constexpr int hop_batch_nt(int prec, int tps) { return prec == TM_F64 ? fx_nt(1) : hop_spb(tps) * tps; }
 constexpr int hop_batch_min_blocks(int prec, int nreal, int tps) {
-  return prec == TM_F64 ? 16 * 32 / fx_nt(1) : (tps == 1 && (prec == TM_F32 || prec == TM_F16)) ? 640 / hop_spb(1) : 1;
+  return prec == TM_F64 ? 16 * 32 / fx_nt(1)
+         : (tps == 1 && (prec == TM_F32 || prec == TM_F16)) ? (nreal == 18 ? 512 : 640) / hop_spb(1) : 1;
 }
 
 template <int PREC, int NREAL, bool HAS_Y, int MODE, int TPS>
