@@ -1180,6 +1180,12 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, c
 tm_status set_error(tm_status st, const char* fmt, ...);
 tm_status cuda_check(cudaError_t e, const char* what);
 
+// Workspace slots: 0..17 CG solver, 22..25 tm_apply_Dh, 26 staged input, 27 staged output,
+// 28 initial-guess work space, 29 contraction partials, 30 chronological-guess scalars,
+// 31 BiCGstab state; 18..20 BiCGstab vectors; 21 staged correlator matrices; 32 the FX form of tm_apply_D's
+// input.
+enum { WS_GAMMA = 21, WS_APPLY_DH = 22, WS_STAGE_IN = 26, WS_STAGE_OUT = 27, WS_X0 = 28, WS_CHRONO = 30, WS_BISTATE = 31, WS_FULL_FX = 32, WS_SLOTS };
+
 }  // namespace tmq
 
 // The lattice object (host side).
@@ -1195,8 +1201,8 @@ struct tm_lattice_s {
   int hop_tps[4][3];        // hopping kernel per form (autotuned): threads per site 1, 2, 4, or TM_HOP_PIPELINED
   int hop_tps_forced[4][3]; // set by tm_set_hop_threads: the tuner keeps hands off
   // work space
-  void* ws[40];             // half-field buffers, allocated on demand
-  size_t ws_bytes[40];
+  void* ws[tmq::WS_SLOTS];       // half-field buffers, allocated on demand
+  size_t ws_bytes[tmq::WS_SLOTS];
   double* partials;         // reduction partials
   size_t partials_count;
   unsigned* counters;       // reduction counters (zeroed)
@@ -1289,11 +1295,6 @@ tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g
                      cudaStream_t s);
 tm_status diag_apply(tm_lattice lat, int prec, void* out, const void* in, int nrhs, double dur, double dui,
                      double dlr, double dli, cudaStream_t s);
-// Workspace slots: 0..17 CG solver, 22..25 tm_apply_Dh, 26 staged input, 27 staged output,
-// 28 initial-guess work space, 29 contraction partials, 30 chronological-guess scalars,
-// 31 BiCGstab state; 18..20 BiCGstab vectors; 21 staged correlator matrices; 32 the FX form of tm_apply_D's
-// input.
-enum { WS_GAMMA = 21, WS_APPLY_DH = 22, WS_STAGE_IN = 26, WS_STAGE_OUT = 27, WS_X0 = 28, WS_CHRONO = 30, WS_BISTATE = 31, WS_FULL_FX = 32 };
 // host-buffer staging through workspace slots
 const void* stage_in(tm_lattice lat, int slot, const void* src, size_t bytes, cudaStream_t s, tm_status* st);
 void* stage_out(tm_lattice lat, int slot, void* dst, size_t bytes, tm_status* st);

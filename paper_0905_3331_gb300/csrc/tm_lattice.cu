@@ -112,7 +112,7 @@ EpiCoef epi_g5_y_plus(double c) {  // g5 (y + c H)
 // ------------------------------------------------------------------ buffers ---
 void* workspace(tm_lattice lat, int slot, size_t bytes, tm_status* st) {
   *st = TM_OK;
-  if (slot < 0 || slot >= 40) {
+  if (slot < 0 || slot >= WS_SLOTS) {
     *st = set_error(TM_ERR_ARG, "internal: workspace slot %d", slot);
     return nullptr;
   }
@@ -598,7 +598,7 @@ tm_status tm_lattice_destroy(tm_lattice lat) {
   cudaFree(lat->U_canon);
   for (int p = 0; p < 4; ++p)
     for (int l = 0; l < 3; ++l) cudaFree(lat->links[p][l]);
-  for (int k = 0; k < 40; ++k) cudaFree(lat->ws[k]);
+  for (int k = 0; k < WS_SLOTS; ++k) cudaFree(lat->ws[k]);
   cudaFree(lat->partials);
   cudaFree(lat->counters);
   cudaFree(lat->gcounters);
