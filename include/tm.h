@@ -107,7 +107,7 @@ size_t tm_half_field_bytes(tm_lattice lat, tm_prec prec);
  * counterpart).  Each output site's 8 hops are shared by 1, 2 or 4 threads (the partial sums
  * are added in a fixed order); more threads per site keep more memory requests in flight on
  * lattices too small to fill the GPU.  With FP64 storage and 18-real links (computed in 64-bit fixed
- * point on the integer units, at more than FP64's accuracy) each of these threads is a pair of lanes,
+ * point on the integer units; accuracy at tm_apply_hopping_eo) each of these threads is a pair of lanes,
  * one per projected spin component.  The value 3 (TM_HOP_PIPELINED, FP32 and FP16 storage
  * only) selects one thread per site whose loads of the next hop are issued before the current
  * hop's arithmetic.  The value 5 (TM_HOP_PAIRED, FP32 and FP16 storage only) selects one thread
@@ -150,7 +150,8 @@ tm_status tm_unpack_half(tm_lattice lat, tm_prec prec, double *dst, const void *
 
 /* out = M(f) in on the full lattice (eq. eo0), or M(f)^dag in if dagger != 0
  * (M^dag = gamma5 M(-f) gamma5).  in, out: canonical full fields, host or device,
- * nrhs x 24 V doubles; out must not overlap in.  Computed in FP64 with 18-real links.
+ * nrhs x 24 V doubles; out must not overlap in.  Computed with 18-real links; accuracy as
+ * tm_apply_hopping_eo with TM_F64.
  * Errors: TM_ERR_NO_GAUGE, TM_ERR_ARG (flavour not +-1, aliasing), TM_ERR_CUDA. */
 tm_status tm_apply_D(tm_lattice lat, double *out, const double *in, int flavour, int dagger,
                      int nrhs, void *stream);
@@ -159,7 +160,13 @@ tm_status tm_apply_D(tm_lattice lat, double *out, const double *in, int flavour,
  * of parity out_parity, from the half field of the other parity (H_eo / H_oe of eq. eo2;
  * M_eo = -kappa H_eo).  in, out: device half fields of precision `prec`, nrhs of them;
  * out must not overlap in.  Links in format `link` (built on first use).  Arithmetic is
- * FP64 for TM_F64 (with 18-real links: 57-bit fixed point) and FP32 otherwise.  The spin projection (1 +- gamma_mu) is applied
+ * FP64 for TM_F64 with 12- and 8-real links, 64-bit fixed point for TM_F64 with 18-real links, and
+ * FP32 otherwise.  The fixed-point sum is off by ~2^-57 of the largest real of the site's eight neighbours
+ * (a site's reals share one exponent) and is then rounded to FP64: closer than FP64 arithmetic in norm, but
+ * a component more than a factor 2^6 below its site's largest enters with fewer bits than FP64 has (59 - k
+ * at 2^-k).  Sites with non-finite reals, or whose largest is below 2^-894 or from 2^978 on, take FP64
+ * arithmetic.  The same holds for tm_apply_D and inside the FP64 solvers; the fields that solvers return
+ * are FP64.  The spin projection (1 +- gamma_mu) is applied
  * before the SU(3) multiply (Sec. 4.1), so each hop multiplies two colour vectors.
  * Errors: TM_ERR_NO_GAUGE, TM_ERR_ARG, TM_ERR_UNSUPPORTED, TM_ERR_CUDA. */
 tm_status tm_apply_hopping_eo(tm_lattice lat, int out_parity, void *out, const void *in,
@@ -357,8 +364,12 @@ tm_status tm_solve_doublet(tm_lattice lat, double *x, const double *b, double mu
  * solution for the source of spin s and colour c.  out: T x 12 x 12 complex doubles (host or
  * device), out[t][j][k] = sum_{x, x_t = t} <psi_j(x), psi_k(x)> (conjugate on psi_j); then
  * C_PG(t) = sum_{s, s', c} out[t][3s+c][3s'+c] (Gamma gamma5)[s'][s], e.g. C_PP(t) = trace.
- * FP64, deterministic; exactly hermitian (the 78 entries j <= k are summed, the others are
- * their conjugates).  Device props must be 16-byte aligned (host props are staged).
+ * Deterministic; exactly hermitian (the 78 entries j <= k are summed, the others are
+ * their conjugates).  Summed in exact integers of the propagators' leading bits: a real of field j is
+ * held to 2^-51 or better of the largest real of field j in the timeslice (mostly of the 1024 components
+ * summed together).  The error of an entry is relative to the two fields' maxima, and below FP64's in
+ * norm.  Non-finite and very small or large reals are summed in FP64.  Were a device wait of the kernel to run out, its
+ * entries would be NaN.  Device props must be 16-byte aligned (host props are staged).
  * Errors: TM_ERR_ARG, TM_ERR_CUDA. */
 tm_status tm_meson_contract(tm_lattice lat, const double *props, double *out, void *stream);
 

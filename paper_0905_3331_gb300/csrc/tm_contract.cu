@@ -21,7 +21,8 @@ namespace tmq {
 // FP64 rate to speak of, so it runs on the fp16 ones with the operands split into exact digits (the
 // scheme of Ozaki, Ogita, Oishi and Rump 2012):
 //   a real is v 2^(E - 1077), v a 55-bit integer (rounded), E one exponent per propagator (at least one
-//   above the largest real of the tiles it serves); v = sum_i d_i 256^(6 - i), seven balanced digits
+//   above the largest real of the tiles it serves, and at most four where it is set anew, so that those
+//   reals keep 51 to 53 bits and smaller ones what lies above the same place); v = sum_i d_i 256^(6 - i), seven balanced digits
 //   -128 <= d_i < 128, each exact in fp16;
 //   sum_k v_r v_c = sum_{i + j <= 7} 256^(12 - i - j) sum_k d_i(r, k) d_j(c, k),
 // every inner sum an integer below 1024 2^14 = 2^24, exact in FP32, over at most CK = 1024 components;

@@ -24,6 +24,10 @@
 // far below the final rounding to FP64.  Measured against 113-bit arithmetic (4^4, 6^3 x 8, 6^3 x 10):
 // relative error of the sum 5.0e-17 on Gaussian fields (FP64 arithmetic: 1.3e-16), 3.9-5.6e-17 on point
 // sources, 5.5e-17 with time slices a factor e^1.5 apart, 6-8e-17 with sites of random size over e^40.
+// These are relative to the norm.  Entry by entry the error is relative to the largest neighbour real: a
+// component 2^-k below its site's largest enters with 59 - k bits (FP64: 53), and not at all from k = 59
+// on.  That shows only where links do not mix colours (unit or diagonal links) or the spins of the other
+// lane stay apart.  12- and 8-real links keep FP64 arithmetic, and so do the fields that solvers return.
 //
 // A neighbour read from an FP64 field that has a non-finite real, or whose largest real is outside
 // [2^-894, 2^978) without being zero throughout, has no FX form (exponent FX_BAD): its output site takes
