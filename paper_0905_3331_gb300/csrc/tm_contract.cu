@@ -473,7 +473,9 @@ extern "C" tm_status tm_meson_contract(tm_lattice lat, const double* props, doub
   const size_t out_bytes = (size_t)T * 12 * 12 * 2 * sizeof(double);
   double* dout = static_cast<double*>(stage_out(lat, WS_STAGE_OUT, out, out_bytes, &st));
   if (st != TM_OK) return st;
-  // two blocks per SM over all timeslices (one wave); each block loops over its tiles
+  // two blocks per SM over all timeslices (one wave); each block loops over its tiles.  Rounded down: above 152
+  // timeslices one block each, which leaves up to half of the slots empty (160 x 12^3 544 us; 48 x 24^3, 2.4 times
+  // the sites, 726)
   const int ntile = (spatial * 12 + CT - 1) / CT;
   const int nbx = std::max(1, std::min(ntile, 2 * 152 / T));
   double* partial =

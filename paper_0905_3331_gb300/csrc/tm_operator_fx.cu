@@ -135,8 +135,9 @@ __global__ void __launch_bounds__(fx_nt(P), HOP_FX_WARPS * 32 / fx_nt(P))
 // (both a few per cent less since the site term's real part became a sign).
 // Small: the launch and the pass over the FX form cost more than converting each neighbour as it is read,
 // eight times over.  The pairs per site are as many as one field fits on the chip in a wave of 16 warps
-// per SM.  With one pair both forms give the same bits, so that a field's result does not depend on the
-// right-hand sides beside it; with more, the canonical form serves any number of them.
+// per SM, so that a field's bits do not depend on the right-hand sides beside it.  With one pair both forms
+// give the same bits; the FX form has no kernel with two or four, so there the canonical form serves any
+// number of fields, also where one pair on the FX form would be quicker (3 fields of 8^3 x 16).
 constexpr size_t CANON_SITES = 65536;
 constexpr size_t WAVE_LANES = 152 * 16 * 32;
 // The FX form of as many fields at a time as fit in 256 MiB (1.4 million sites), at least one.  Smaller chunks
