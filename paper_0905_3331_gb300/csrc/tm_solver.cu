@@ -748,12 +748,11 @@ tm_status cg_normal(const Solver& S, const tm_cg_params& P, const void* bp, doub
   bool converged = false;
   double rr_true = bb;
   // starting residual R = b' - A X (X = 0 unless a guess is given)
-  bool w_valid = false;  // W = Qhat^{-f} X of the current X (K2 of the last FP64 residual)
-  // FP64 mode: its last residual leaves x_o.  The mixed modes recompute it when they return it: an FP64 W
-  // costs their residuals ~30 % of K3 each.
-  const bool keep_w = P.mode == TM_CG_FP64;
+  // W = Qhat^{-f} X of the current X in FP64 (K2 of the last FP64 residual).  Kept by the residuals that may end
+  // the solve; a reliable update's would be ~30 % slower in K3, and x_o is formed anew after it.
+  bool w_valid = false;
   if (guess) {
-    if ((st = true_residual(S, R, X, bp, T, W, &rr_true, keep_w)) != TM_OK) return st;
+    if ((st = true_residual(S, R, X, bp, T, W, &rr_true, true)) != TM_OK) return st;
     w_valid = true;
   } else {
     if ((st = cuda_check(cudaMemsetAsync(X, 0, S.hb[TM_F64], s), "memset")) != TM_OK) return st;
@@ -778,7 +777,7 @@ tm_status cg_normal(const Solver& S, const tm_cg_params& P, const void* bp, doub
       if (fin.nonfinite) return set_error(TM_ERR_NONFINITE, "tm_solve_cg: non-finite value in the iteration");
       const bool progress = fin.iter > iters;
       iters = fin.iter;
-      if ((st = true_residual(S, R, X, bp, T, W, &rr_true, keep_w)) != TM_OK) return st;
+      if ((st = true_residual(S, R, X, bp, T, W, &rr_true, true)) != TM_OK) return st;
       w_valid = true;
       ++updates;
       trace_update(updates, rr_true, bb);
@@ -836,7 +835,7 @@ tm_status cg_normal(const Solver& S, const tm_cg_params& P, const void* bp, doub
         count_launch();
         w_valid = false;
       }
-      if ((st = true_residual(S, R, X, bp, T, W, &rr_true, keep_w)) != TM_OK) return st;
+      if ((st = true_residual(S, R, X, bp, T, W, &rr_true, true)) != TM_OK) return st;
       w_valid = true;
       ++updates;
       trace_update(updates, rr_true, bb);
@@ -935,8 +934,8 @@ tm_status cg_normal(const Solver& S, const tm_cg_params& P, const void* bp, doub
         rsrc = Rd;
         rprec = TM_DF64;
       } else {
-        if ((st = true_residual(S, R, X, bp, T, W, &rr_true, keep_w)) != TM_OK) return st;
-        w_valid = true;
+        if ((st = true_residual(S, R, X, bp, T, W, &rr_true, false)) != TM_OK) return st;
+        w_valid = false;
       }
       ++updates;
       trace_update(updates, rr_true, bb);
@@ -946,7 +945,7 @@ tm_status cg_normal(const Solver& S, const tm_cg_params& P, const void* bp, doub
           break;
         }
         // confirm in FP64; if the double-float residual was too optimistic, carry on in FP64
-        if ((st = true_residual(S, R, X, bp, T, W, &rr_true, keep_w)) != TM_OK) return st;
+        if ((st = true_residual(S, R, X, bp, T, W, &rr_true, true)) != TM_OK) return st;
         w_valid = true;
         ++updates;
         trace_update(updates, rr_true, bb);
@@ -973,7 +972,7 @@ tm_status cg_normal(const Solver& S, const tm_cg_params& P, const void* bp, doub
   res->updates = updates;
   res->converged = converged;
   res->rr_true = rr_true;
-  res->xo_in_W = w_valid && keep_w;
+  res->xo_in_W = w_valid;
   res->pending = false;
   return TM_OK;
 }
