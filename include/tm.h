@@ -395,8 +395,9 @@ void tm_cg_params_default(tm_cg_params *params);
  * device-memory budget (a framework whose caching allocator already holds the memory, a
  * process with a hard memory limit) or in a latency-critical loop where a cudaMalloc or
  * cudaFree would synchronise the device.  tm_apply_D takes its work buffer
- * (up to 256 MiB, or one field's if that is more; none on lattices of up to 19456 sites) from
- * lattice-owned memory allocated on first use, once, whatever nrhs is; this variant takes it from one static
+ * (up to 256 MiB, or one field's if that is more; only calls on more than 65536 sites, fields
+ * included, and lattices of more than 19456 need it) from lattice-owned memory allocated on first
+ * use outside a stream capture, once, whatever nrhs is; this variant takes it from one static
  * 64 MiB device array that is part of the library's device code, so the call itself calls no
  * cudaMalloc, cudaFree or other allocating routine.  Every GPU that loads the library holds
  * those 64 MiB until the process exits.

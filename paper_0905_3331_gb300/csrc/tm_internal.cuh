@@ -1287,10 +1287,10 @@ bool hop_tps_fixed(tm_lattice lat, int prec, int nreal);
 
 // out = M(f) in (eq. eo0), or gamma5 M(f) gamma5 in with g5, on canonical FP64 device fields (nrhs of them);
 // scratch holds the FX form of `per` fields at a time, full_fx_bytes(h) each (tm_operator_fx.cu; few sites
-// are not brought to it)
+// are not brought to it, nor any with per = 0)
 inline size_t full_fx_bytes(size_t h) { return (2 * fx_field_bytes(h) + 255) / 256 * 256; }
-// fields of the scratch that serves any nrhs, 0 if none needs one (once the FP64 links are built)
-int full_fx_fields(tm_lattice lat);
+// fields of the scratch that serves any nrhs, 0 if this one needs none (once the FP64 links are built)
+int full_fx_fields(tm_lattice lat, int nrhs);
 tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g5, int nrhs, void* scratch, int per,
                      cudaStream_t s);
 tm_status diag_apply(tm_lattice lat, int prec, void* out, const void* in, int nrhs, double dur, double dui,

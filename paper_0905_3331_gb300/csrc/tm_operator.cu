@@ -56,7 +56,12 @@ tm_status tm_apply_D(tm_lattice lat, double* out, const double* in, int flavour,
   // the FX form of a fixed number of fields, whatever nrhs is: a buffer sized by nrhs would be freed and
   // allocated anew by a call with more of them, under the feet of a captured one
   if ((st = ensure_links(lat, TM_F64, 18, s)) != TM_OK) return st;
-  const int per = full_fx_fields(lat);
+  int per = full_fx_fields(lat, nrhs);
+  if (per > 0 && lat->ws[WS_FULL_FX] == nullptr) {  // nothing is allocated in a capture: the form without a buffer, same bits
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+    if (cap != cudaStreamCaptureStatusNone) per = 0;
+  }
   void* w = nullptr;
   if (per > 0) w = workspace(lat, WS_FULL_FX, full_fx_bytes(lat->h) * per, &st);
   if (st != TM_OK) return st;

@@ -151,8 +151,10 @@ static int full_pairs(tm_lattice lat) {
   return lat->V * 8 <= WAVE_LANES ? 4 : (lat->V * 4 <= WAVE_LANES ? 2 : 1);
 }
 
-int full_fx_fields(tm_lattice lat) {
-  return full_pairs(lat) > 1 ? 0 : (int)std::max<size_t>(1, FULL_FX_BYTES / full_fx_bytes(lat->h));
+int full_fx_fields(tm_lattice lat, int nrhs) {
+  return full_pairs(lat) > 1 || (size_t)std::min(nrhs, MAX_FIELDS) * lat->V <= CANON_SITES
+             ? 0
+             : (int)std::max<size_t>(1, FULL_FX_BYTES / full_fx_bytes(lat->h));
 }
 
 tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g5, int nrhs, void* scratch, int per,
@@ -179,7 +181,7 @@ tm_status apply_full(tm_lattice lat, double* out, const double* in, int f, int g
   const int pairs = full_pairs(lat);
   for (int r = 0, n; r < nrhs; r += n) {
     n = std::min(nrhs - r, MAX_FIELDS);
-    const bool canon = pairs > 1 || (size_t)n * lat->V <= CANON_SITES;
+    const bool canon = per == 0 || pairs > 1 || (size_t)n * lat->V <= CANON_SITES;
     if (!canon) n = (n + (n + per - 1) / per - 1) / ((n + per - 1) / per);  // equal chunks of at most `per`
     const double* src = in + (size_t)r * lat->V * 24;
     double* dst = out + (size_t)r * lat->V * 24;

@@ -55,6 +55,25 @@ def test_captured_call_before_more_fields():
         assert torch.equal(y[0], z[0]) and torch.equal(w, z)
 
 
+def test_capture_before_the_buffer_exists():
+    """Two fields of 54880 sites need the buffer, one does not: captured first, they do without."""
+    T, L = 20, 14
+    with lattice(T, L) as lat:
+        x = fields(2, T, L)
+        y, z = torch.zeros_like(x), torch.zeros_like(x)
+        s = torch.cuda.Stream()
+        s.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(s):
+            lat.apply_D(z[:1], x[:1])
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=s):
+                lat.apply_D(y, x, nrhs=2)
+            g.replay()
+            lat.apply_D(z, x, nrhs=2)
+        torch.cuda.synchronize()
+        assert torch.equal(y, z)
+
+
 @pytest.mark.parametrize("threads", [0, 1])
 def test_more_fields_than_a_grid_dimension(threads):
     """65600 fields on 2^4 against the same fields in three calls."""
